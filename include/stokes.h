@@ -109,11 +109,12 @@ typedef struct {
                             M_Q, L_Q on levels with >= 2^18 rows, CSR below; the
                             strain-form A in symmetric stencil storage (diagonal
                             and upper 3x3 blocks only: half the matrix bytes)
-                            for its products and the double-float refinement
-                            residual;
+                            for its FP64 products and the double-float
+                            refinement residual, its FP32 products element by
+                            element from the tetrahedra's geometry;
                             1: CSR everywhere (A as BSR3, CSR of 3x3 blocks);
                             2: stencil storage on every level, A as in 0;
-                            3: as 0 but the products of A from BSR3 (the
+                            3: as 0 but all products of A from BSR3 (the
                             refinement residual still symmetric) */
   int graphs;            /* 1 (default): V-cycles, and C when schur_inner_iters
                             > 0, are recorded into CUDA graphs on a private
@@ -153,7 +154,7 @@ typedef struct {
                             An interval far below the spectrum makes the
                             V-cycle indefinite; the Krylov solvers then report
                             STOKES_ERR_BREAKDOWN. */
-  int sym_batch;         /* symmetric A products: block entries whose loads one
+  int sym_batch;         /* symmetric (FP64) A products: block entries whose loads one
                             thread issues before using them (2, 4 or 8; 0:
                             default 8) */
   int stencil_min_rows;  /* formats 0 and 3: levels with at least this many rows
@@ -277,6 +278,9 @@ typedef enum {
                                  residual computes it: FP32 hi/lo pairs of A
                                  and x, exact FP32 products, double-float sums
                                  (mixed-precision contexts only)              */
+  STOKES_OP_A_F32 = 19,       /* y = A x as the FP32 inner solves compute it:
+                                 x rounded to FP32 (mixed-precision contexts
+                                 only)                                        */
   STOKES_OP_VCYCLE_VEL = 18   /* y = the configured velocity preconditioner
                                  (vcycles V-cycles of A~_{vel_prec}) applied
                                  to x, from level 0                          */
@@ -332,7 +336,7 @@ stokes_status stokes_sizes(stokes_ctx* ctx, int64_t sizes[6]);
  * (matrix read once, each vector read/written once) since the last reset. */
 typedef enum {
   STOKES_KERNEL_SPMM_A3 = 0,      /* A~_3 x 3 RHS on the finest level (smoother/residual) */
-  STOKES_KERNEL_SPMV_A = 1,       /* BSR3 strain-form A                     */
+  STOKES_KERNEL_SPMV_A = 1,       /* products of the strain-form A          */
   STOKES_KERNEL_B = 2,            /* divergence B                           */
   STOKES_KERNEL_BT = 3,           /* gradient B^T                           */
   STOKES_KERNEL_SPMV_P1 = 4,      /* P1 CSR (M_Q, L_Q, eps M_Q + L_Q)       */

@@ -257,18 +257,31 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
   }
   if (c.opt.format != 1) {
     // the strain-form A also in symmetric stencil storage (half the values, no
-    // indices): every product of A reads it (48^3, FP32, with the fused dot:
-    // 171 us against 243 us for BSR3), and the double-float refinement
-    // residual (324 against 421 us); format 3 keeps BSR3 for the products
+    // indices) for its FP64 products and the double-float refinement residual
+    // (48^3: 324 against 421 us for BSR3); FP32 products are formed element by
+    // element (48^3 with the fused dot: 40 us against 165 us for the symmetric
+    // storage and 243 us for BSR3); format 3 keeps BSR3 for the products
     c.symA.reset(sym3_from_csr(c.ex, c.arena, st, n, c.A));
     c.A.sym = c.symA.get();
     c.A.sym_products = c.opt.format != 3;
+    if (c.mixed && c.A.sym_products) {
+      c.elA = std::make_unique<ElementOp>();
+      c.elA->n = n;
+      c.elA->mu = (float)c.mu;
+      c.elA->G = element_geometry(c.ex, c.arena, n, c.lv[0].X, c.dt);
+      // four right-hand sides per launch while their partial sums stay in L2
+      const size_t one = element_part_words(n);
+      c.elA->batch = kFusedDots * sizeof(float) * one <= ((size_t)64 << 20) ? kFusedDots : 1;
+      c.elA->part = c.arena.alloc<float>(c.elA->batch * one);
+      c.A.el = c.elA.get();
+    }
   }
   // per-block partials of dot products fused into other kernels
   c.ds.fused_cap = std::max(std::max(kDotBlocks * kMaxBasis, bsr3_dot_grid(c.A)), c.symA ? sym3_grid(*c.symA) : 0);
+  c.ds.fused_cap = std::max(c.ds.fused_cap, c.elA ? element_dot_grid(n) : 0);
   c.ds.fused_partial = c.arena.alloc<double>(c.ds.fused_cap);
-  c.ds.fused_counter = c.arena.alloc<unsigned>(1);
-  SK_CUDA(cudaMemsetAsync(c.ds.fused_counter, 0, sizeof(unsigned), c.ex.s));
+  c.ds.fused_counter = c.arena.alloc<unsigned>(kFusedDots);
+  SK_CUDA(cudaMemsetAsync(c.ds.fused_counter, 0, sizeof(unsigned) * kFusedDots, c.ex.s));
   c.ds.k_cap = kdot_scratch(3 * (size_t)c.lv[0].nvi + c.lv[0].np, kMaxRhs);
   c.ds.k_partial = c.arena.alloc<double>((size_t)c.ds.k_cap);
   c.ds.k_counter = c.arena.alloc<unsigned>(kMaxRhs);

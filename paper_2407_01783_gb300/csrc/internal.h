@@ -278,6 +278,17 @@ template <> inline float* Sym3Op::v<float>() const { return v32; }
 // br*bc planes of nnz entries each (plane j at v + j*nnz) so that consecutive
 // lanes read consecutive addresses.
 // ---------------------------------------------------------------------------
+// The strain-form A of one level evaluated element by element in FP32
+// (element.cu): per-tetrahedron geometry and the work space of one product.
+constexpr int kElWords = 12;  // geometry words per tetrahedron
+struct ElementOp {
+  int n = 0;
+  float mu = 0;
+  const float* G = nullptr;  // geometry records
+  float* part = nullptr;     // [batch][element_part_words] partial sums of the cubes
+  int batch = 1;             // right-hand sides per launch
+};
+
 struct Csr {
   int rows = 0, cols = 0;
   long long nnz = 0;
@@ -295,6 +306,7 @@ struct Csr {
   const Sym3Op* sym = nullptr;    // 3x3-block matrix in symmetric stencil storage: used for the
                                   // double-float residual, and for all products if sym_products
   bool sym_products = false;
+  const ElementOp* el = nullptr;  // FP32 products element by element instead (with sym_products)
   template <class T> T* v() const;
   double bytes(int elem) const {  // algorithmic bytes of one product (matrix only)
     return (double)nnz * (4.0 + elem * br * bc) + 4.0 * (rows + 1);
@@ -560,7 +572,7 @@ struct DotScratch {
   // dot products fused into the epilogue of another kernel: one partial per
   // block of that launch (capacity fused_cap), own completion counter
   double* fused_partial = nullptr;
-  unsigned* fused_counter = nullptr;
+  unsigned* fused_counter = nullptr;  // kFusedDots of them (one per right-hand side of a launch)
   int fused_cap = 0;
   // dot products of K right-hand sides (multi.cu): partials [K][vectors][blocks]
   // and one completion counter per (right-hand side, vector)
@@ -606,17 +618,21 @@ __device__ __forceinline__ void grid_sum(double v, double* partial, unsigned* co
 }
 #endif
 constexpr int kMaxDots = 4;
+constexpr int kFusedDots = 4;
 constexpr int kDotBlocks = 608;  // 4 x 152 SMs
 // y = A x, and *dot = x . y (deterministic, FP64 accumulation) fused into the
 // same kernel when A has symmetric stencil storage (else a separate dot).
 template <class T> bool bsr3_apply_dot(const Exec& ex, const Csr& m, const T* x, T* y, const DotScratch& ds,
                                        double* dot);
-// symmetric-stencil products (sym3.cu): y = A x or y = b - A x, optional fused
+// the same for k right-hand sides [k][3][rows]: dot[i] = x_i . (A x_i)
+template <class T> void bsr3_apply_dot_k(const Exec& ex, const Csr& m, int k, const T* x, T* y, const DotScratch& ds,
+                                         double* dot);
+// symmetric-stencil products (sym3.cu, FP64): y = A x or y = b - A x, optional fused
 // dot x . (A x); double-float residual y = b - A x
-template <class T> void sym3_launch(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, const DotScratch* ds,
-                                    double* dot);
+void sym3_launch(const Exec& ex, const Csr& m, const double* x, double* y, const double* b, const DotScratch* ds,
+                 double* dot);
 // the same (no dot) for four right-hand sides [4][3][rows] in one sweep
-template <class T> void sym3_launch4(const Exec& ex, const Csr& m, const T* x, T* y, const T* b);
+void sym3_launch4(const Exec& ex, const Csr& m, const double* x, double* y, const double* b);
 // k right-hand sides of the BSR3 operator (x, y, b: [k][3][rows]): one sweep
 // for k = 4 with symmetric storage, else one product per right-hand side
 template <class T> void bsr3_apply_k(const Exec& ex, const Csr& m, int k, const T* x, T* y, const T* b,
@@ -624,6 +640,13 @@ template <class T> void bsr3_apply_k(const Exec& ex, const Csr& m, int k, const 
 void sym3_residual_df(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y);
 // the same for four right-hand sides [4][3][rows] in one sweep
 void sym3_residual_df4(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y);
+// element-by-element FP32 products (element.cu): y = A x or y = b - A x for k
+// right-hand sides [k][3][rows]; with dot, dot[q] = x_q . (A x_q)
+float* element_geometry(const Exec& ex, Arena& ar, int n, const double* X, double dt);
+size_t element_part_words(int n);  // work space of one right-hand side
+int element_dot_grid(int n);  // blocks of a dot-fused launch (all right-hand sides)
+void element_strain(const Exec& ex, const ElementOp& e, int k, const float* x, float* y, const float* b,
+                    const DotScratch* ds, double* dot);
 double sym3_bytes(const Sym3Op& so, int esz, int rows, int streams);
 // most blocks of one symmetric-stencil product launch (fused-dot partial capacity)
 int sym3_grid(const Sym3Op& so);
@@ -808,6 +831,7 @@ struct stokes_ctx {
   // last forward solution (reduced) for the adjoint
   std::vector<std::unique_ptr<sk::StencilOp>> stencils;  // owned stencil storages
   std::unique_ptr<sk::Sym3Op> symA;                       // A in symmetric stencil storage
+  std::unique_ptr<sk::ElementOp> elA;                     // A element by element (mixed precision)
   double* U_last = nullptr;
   double* P_last = nullptr;
   bool have_solution = false;

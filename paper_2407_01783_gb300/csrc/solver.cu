@@ -1333,7 +1333,7 @@ template <class T> static int ainv_k(stokes_ctx& c, int K, const T* t, T* w, dou
           op_A_k<T>(c, K, x, y);
           kdot<T>(c.ex, c.ds, nv, 0, K, 1, x, (const T*)y, dq);
         } else {
-          for (int k = 0; k < K; ++k) bsr3_apply_dot<T>(c.ex, c.A, x + k * nv, y + k * nv, c.ds, dq + k);
+          bsr3_apply_dot_k<T>(c.ex, c.A, K, x, y, c.ds, dq);
         }
       },
       [&](const T* r, T* z) { vcycles<T>(c, velocity_cycle(c), r, z, std::max(1, c.opt.vcycles), K); }, t, w, tol,
@@ -2016,6 +2016,14 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       Tmp<double> t(c.pool, nv);
       bsr3_residual_df(c.ex, c.A, xh, xl, zero_b, t, STOKES_KERNEL_RESIDUAL);  // t = -A x
       scale_copy<double>(c.ex, nv, Coef::constant(-1.0), t, y);
+      break;
+    }
+    case STOKES_OP_A_F32: {
+      SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 A needs a mixed-precision context");
+      Tmp<float> xf(c.pool, nv), yf(c.pool, nv);
+      convert<double, float>(c.ex, nv, x, xf);
+      bsr3_apply<float>(c.ex, c.A, xf, yf, (const float*)nullptr);
+      convert<float, double>(c.ex, nv, yf, y);
       break;
     }
     default: throw Error(STOKES_ERR_ARG, "unknown operator");

@@ -1024,11 +1024,30 @@ template <class T> void bsr3_cheb(const Exec& ex, const Csr& m, const T* b, cons
   ProfScope ps(ex, kind, prod_bytes(m, sizeof(T), 3, 3, 4) + 3.0 * sizeof(T) * m.rows);
   launch(ex, m, SH_BSR3, xin, EpiCheb3<T>{b, xin, d, xout, dinv, (T)c1, (T)c2, (size_t)m.rows}, m.group);
 }
+// FP32 products of A run element by element (element.cu) wherever the context
+// has the geometry (mixed precision, formats 0 and 2): faster than the stored
+// blocks on every mesh measured, 8^3 to 96^3 (figures there)
+template <class T> static inline bool use_element(const Csr& m) {
+  return std::is_same<T, float>::value && m.el && m.sym_products;
+}
+// geometry once, x gathered once, y and `streams` further vectors once
+static double element_bytes(const ElementOp& e, int rows, int k, int streams) {
+  return 4.0 * (6.0 * kElWords * e.n * e.n * e.n + 3.0 * rows * k * (2 + streams));
+}
 template <class T> void bsr3_apply(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, int kind) {
-  if (m.sym && m.sym->template v<T>() && m.sym_products) {
-    ProfScope ps(ex, kind, sym3_bytes(*m.sym, sizeof(T), m.rows, b ? 1 : 0));
-    sym3_launch<T>(ex, m, x, y, b, nullptr, nullptr);
-    return;
+  if constexpr (std::is_same<T, float>::value) {
+    if (use_element<T>(m)) {
+      ProfScope ps(ex, kind, element_bytes(*m.el, m.rows, 1, b ? 1 : 0));
+      element_strain(ex, *m.el, 1, x, y, b, nullptr, nullptr);
+      return;
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    if (m.sym && m.sym_products) {
+      ProfScope ps(ex, kind, sym3_bytes(*m.sym, sizeof(T), m.rows, b ? 1 : 0));
+      sym3_launch(ex, m, x, y, b, nullptr, nullptr);
+      return;
+    }
   }
   ProfScope ps(ex, kind, prod_bytes(m, sizeof(T), 3, 3, b ? 1 : 0));
   if (b) launch(ex, m, SH_BSR3, x, EpiResid<T, 3>{b, y, (size_t)m.rows}, m.group);
@@ -1036,21 +1055,39 @@ template <class T> void bsr3_apply(const Exec& ex, const Csr& m, const T* x, T* 
 }
 template <class T>
 void bsr3_apply_k(const Exec& ex, const Csr& m, int k, const T* x, T* y, const T* b, int kind) {
-  if (k == 4 && m.sym && m.sym->template v<T>() && m.sym_products) {
-    ProfScope ps(ex, kind, (double)m.sym->total * sizeof(T) + (double)sizeof(T) * 3.0 * m.rows * 4 * (b ? 2 : 1));
-    sym3_launch4<T>(ex, m, x, y, b);
-    return;
+  if constexpr (std::is_same<T, float>::value) {
+    if (use_element<T>(m)) {
+      ProfScope ps(ex, kind, element_bytes(*m.el, m.rows, k, b ? 1 : 0));
+      element_strain(ex, *m.el, k, x, y, b, nullptr, nullptr);
+      return;
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    if (k == 4 && m.sym && m.sym_products) {
+      ProfScope ps(ex, kind, (double)m.sym->total * sizeof(T) + (double)sizeof(T) * 3.0 * m.rows * 4 * (b ? 2 : 1));
+      sym3_launch4(ex, m, x, y, b);
+      return;
+    }
   }
   const size_t len = 3 * (size_t)m.rows;
   for (int i = 0; i < k; ++i) bsr3_apply<T>(ex, m, x + i * len, y + i * len, b ? b + i * len : nullptr, kind);
 }
 template <class T> bool bsr3_apply_dot(const Exec& ex, const Csr& m, const T* x, T* y, const DotScratch& ds,
                                        double* dot) {
-  if (m.sym && m.sym->template v<T>() && m.sym_products && ds.fused_partial && sym3_grid(*m.sym) <= ds.fused_cap) {
-    // the product's bytes plus the own-row x read of the fused dot
-    ProfScope ps(ex, STOKES_KERNEL_SPMV_A, sym3_bytes(*m.sym, sizeof(T), m.rows, 1));
-    sym3_launch<T>(ex, m, x, y, (const T*)nullptr, &ds, dot);
-    return true;
+  if constexpr (std::is_same<T, float>::value) {
+    if (use_element<T>(m)) {
+      ProfScope ps(ex, STOKES_KERNEL_SPMV_A, element_bytes(*m.el, m.rows, 1, 1));
+      element_strain(ex, *m.el, 1, x, y, nullptr, &ds, dot);
+      return true;
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    if (m.sym && m.sym_products && ds.fused_partial && sym3_grid(*m.sym) <= ds.fused_cap) {
+      // the product's bytes plus the own-row x read of the fused dot
+      ProfScope ps(ex, STOKES_KERNEL_SPMV_A, sym3_bytes(*m.sym, sizeof(T), m.rows, 1));
+      sym3_launch(ex, m, x, y, (const T*)nullptr, &ds, dot);
+      return true;
+    }
   }
   if (m.template v<T>() && ds.fused_partial && bsr3_dot_grid(m) <= ds.fused_cap) {
     ProfScope ps(ex, STOKES_KERNEL_SPMV_A, prod_bytes(m, sizeof(T), 3, 3, 1));
@@ -1069,6 +1106,19 @@ template <class T> bool bsr3_apply_dot(const Exec& ex, const Csr& m, const T* x,
   const T* ys[1] = {y};
   dots<T>(ex, ds, 1, xs, ys, (size_t)m.rows * 3, dot, kDotFast);
   return false;
+}
+
+template <class T>
+void bsr3_apply_dot_k(const Exec& ex, const Csr& m, int k, const T* x, T* y, const DotScratch& ds, double* dot) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (use_element<T>(m)) {
+      ProfScope ps(ex, STOKES_KERNEL_SPMV_A, element_bytes(*m.el, m.rows, k, 1));
+      element_strain(ex, *m.el, k, x, y, nullptr, &ds, dot);
+      return;
+    }
+  }
+  const size_t len = 3 * (size_t)m.rows;
+  for (int i = 0; i < k; ++i) bsr3_apply_dot<T>(ex, m, x + i * len, y + i * len, ds, dot + i);
 }
 
 template <class T> void b_apply(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, double alpha, int k) {
@@ -1258,7 +1308,8 @@ void autotune_group(const Exec& ex, Csr& m, int nr, int kind, int k) {
   template void bt_apply<T>(const Exec&, const Csr&, const T*, T*, const T*, const T*, double, int);     \
   template void dense_apply<T>(const Exec&, const T*, int, int, const T*, T*, bool);                    \
   template void bsr3_apply_k<T>(const Exec&, const Csr&, int, const T*, T*, const T*, int);            \
-  template bool bsr3_apply_dot<T>(const Exec&, const Csr&, const T*, T*, const DotScratch&, double*);
+  template bool bsr3_apply_dot<T>(const Exec&, const Csr&, const T*, T*, const DotScratch&, double*);   \
+  template void bsr3_apply_dot_k<T>(const Exec&, const Csr&, int, const T*, T*, const DotScratch&, double*);
 SK_INST(float)
 SK_INST(double)
 

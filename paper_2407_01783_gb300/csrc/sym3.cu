@@ -338,9 +338,9 @@ double sym3_bytes(const Sym3Op& so, int esz, int rows, int streams) {
   return (double)so.total * esz + (double)esz * 3.0 * rows * (1 + streams);
 }
 
-template <int G, int U, class T>
-static void sym3_launch_g(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, const DotScratch* ds,
-                          double* dot) {
+template <int G, int U>
+static void sym3_launch_g(const Exec& ex, const Csr& m, const double* x, double* y, const double* b,
+                          const DotScratch* ds, double* dot) {
   const Sym3Op& so = *m.sym;
   const Sym3Args a = sym3_args(so, G);
   const int nvb = sym3_blocks(so, a);
@@ -353,17 +353,17 @@ static void sym3_launch_g(const Exec& ex, const Csr& m, const T* x, T* y, const 
     int dev = 0, sms = 0, occ = 0;
     SK_CUDA(cudaGetDevice(&dev));
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (dot) SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, T, true>, kSymBlock, 0));
-    else SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, T, false>, kSymBlock, 0));
+    if (dot) SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, double, true>, kSymBlock, 0));
+    else SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, double, false>, kSymBlock, 0));
     w = std::max(1, sms * std::max(1, occ));
   }
   const int grid = std::min(nvb, w);
   if (dot) {
     SK_REQUIRE(ds && ds->fused_partial && grid <= ds->fused_cap, STOKES_ERR_ARG, "fused dot scratch too small");
-    k_sym3<G, U, T, true><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.template v<T>(), x, (size_t)m.rows, b, y,
+    k_sym3<G, U, double, true><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y,
                                                     ds->fused_partial, ds->fused_counter, dot);
   } else {
-    k_sym3<G, U, T, false><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.template v<T>(), x, (size_t)m.rows, b, y, nullptr,
+    k_sym3<G, U, double, false><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
                                                      nullptr, nullptr);
   }
   SK_CHECK_LAUNCH();
@@ -371,7 +371,7 @@ static void sym3_launch_g(const Exec& ex, const Csr& m, const T* x, T* y, const 
 
 // four right-hand sides (x, y, b: [4][3][rows]): every stored block read once
 // for the four; one thread per row, two entries' loads in flight
-template <class T> void sym3_launch4(const Exec& ex, const Csr& m, const T* x, T* y, const T* b) {
+void sym3_launch4(const Exec& ex, const Csr& m, const double* x, double* y, const double* b) {
   const Sym3Op& so = *m.sym;
   const Sym3Args a = sym3_args(so, 1);
   const int nvb = sym3_blocks(so, a);
@@ -381,26 +381,26 @@ template <class T> void sym3_launch4(const Exec& ex, const Csr& m, const T* x, T
     int dev = 0, sms = 0, occ = 0;
     SK_CUDA(cudaGetDevice(&dev));
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<1, 2, T, false, 4>, kSymBlock, 0));
+    SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<1, 2, double, false, 4>, kSymBlock, 0));
     w = std::max(1, sms * std::max(1, occ));
   }
   const int grid = std::min(nvb, w);
-  k_sym3<1, 2, T, false, 4><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.template v<T>(), x, (size_t)m.rows, b, y, nullptr,
+  k_sym3<1, 2, double, false, 4><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
                                                        nullptr, nullptr);
   SK_CHECK_LAUNCH();
 }
 
-template <class T>
-void sym3_launch(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, const DotScratch* ds, double* dot) {
+void sym3_launch(const Exec& ex, const Csr& m, const double* x, double* y, const double* b, const DotScratch* ds,
+                 double* dot) {
   // (threads per row, entries in flight per lane)
   const int g = m.sym->group, u = m.sym->batch;
-  if (g == 1 && u == 2) sym3_launch_g<1, 2, T>(ex, m, x, y, b, ds, dot);
-  else if (g == 1 && u == 4) sym3_launch_g<1, 4, T>(ex, m, x, y, b, ds, dot);
-  else if (g == 1) sym3_launch_g<1, 8, T>(ex, m, x, y, b, ds, dot);
-  else if (g == 2 && u == 2) sym3_launch_g<2, 2, T>(ex, m, x, y, b, ds, dot);
-  else if (g == 2) sym3_launch_g<2, 4, T>(ex, m, x, y, b, ds, dot);
-  else if (g == 4) sym3_launch_g<4, 2, T>(ex, m, x, y, b, ds, dot);
-  else sym3_launch_g<8, 1, T>(ex, m, x, y, b, ds, dot);
+  if (g == 1 && u == 2) sym3_launch_g<1, 2>(ex, m, x, y, b, ds, dot);
+  else if (g == 1 && u == 4) sym3_launch_g<1, 4>(ex, m, x, y, b, ds, dot);
+  else if (g == 1) sym3_launch_g<1, 8>(ex, m, x, y, b, ds, dot);
+  else if (g == 2 && u == 2) sym3_launch_g<2, 2>(ex, m, x, y, b, ds, dot);
+  else if (g == 2) sym3_launch_g<2, 4>(ex, m, x, y, b, ds, dot);
+  else if (g == 4) sym3_launch_g<4, 2>(ex, m, x, y, b, ds, dot);
+  else sym3_launch_g<8, 1>(ex, m, x, y, b, ds, dot);
 }
 
 template <int G>
@@ -431,12 +431,5 @@ void sym3_residual_df(const Exec& ex, const Csr& m, const float* xh, const float
     default: sym3_df_g<4>(ex, m, xh, xl, b, y); break;
   }
 }
-
-template void sym3_launch<float>(const Exec&, const Csr&, const float*, float*, const float*, const DotScratch*,
-                                 double*);
-template void sym3_launch4<float>(const Exec&, const Csr&, const float*, float*, const float*);
-template void sym3_launch4<double>(const Exec&, const Csr&, const double*, double*, const double*);
-template void sym3_launch<double>(const Exec&, const Csr&, const double*, double*, const double*, const DotScratch*,
-                                  double*);
 
 }  // namespace sk
