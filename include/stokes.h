@@ -281,6 +281,8 @@ typedef enum {
   STOKES_OP_A_F32 = 19,       /* y = A x as the FP32 inner solves compute it:
                                  x rounded to FP32 (mixed-precision contexts
                                  only)                                        */
+  STOKES_OP_B_F32 = 20,       /* y = B x, likewise                            */
+  STOKES_OP_BT_F32 = 21,      /* y = B^T x, likewise                          */
   STOKES_OP_VCYCLE_VEL = 18   /* y = the configured velocity preconditioner
                                  (vcycles V-cycles of A~_{vel_prec}) applied
                                  to x, from level 0                          */

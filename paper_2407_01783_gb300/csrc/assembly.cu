@@ -100,6 +100,13 @@ StencilTables* stencils_create(Arena& ar) {
   return st;
 }
 
+void div_offsets(const StencilTables* st, signed char (*d)[3]) {
+  const int b = st->beg[PAT_P1P2][0];
+  SK_REQUIRE(st->beg[PAT_P1P2][1] - b == kDivS, STOKES_ERR_ARG, "unexpected divergence stencil");
+  for (int e = 0; e < kDivS; ++e)
+    for (int c = 0; c < 3; ++c) d[e][c] = (signed char)st->h_off[3 * (b + e) + c];
+}
+
 // Index spaces on the half-grid: q = lo + step * i, 0 <= i < ext per axis.
 struct Space {
   int lo, step, ext;

@@ -276,6 +276,10 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
       c.A.el = c.elA.get();
     }
   }
+  if (c.opt.format != 1) {
+    c.divB.reset(div_from_csr(c.ex, c.arena, st, n, c.B));
+    c.B.div = c.Bt.div = c.divB.get();
+  }
   // per-block partials of dot products fused into other kernels
   c.ds.fused_cap = std::max(std::max(kDotBlocks * kMaxBasis, bsr3_dot_grid(c.A)), c.symA ? sym3_grid(*c.symA) : 0);
   c.ds.fused_cap = std::max(c.ds.fused_cap, c.elA ? element_dot_grid(n) : 0);
@@ -329,8 +333,12 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
     c.A.v32 = f32_copy(c, c.A.v64, 9 * (size_t)c.A.nnz);
     c.A.v32lo = c.arena.alloc<float>(9 * (size_t)c.A.nnz);
     to_f32_lo(c.ex, c.A.v64, c.A.v32, c.A.v32lo, 9 * (size_t)c.A.nnz);
-    c.B.v32 = f32_copy(c, c.B.v64, 3 * (size_t)c.B.nnz);
-    c.Bt.v32 = f32_copy(c, c.Bt.v64, 3 * (size_t)c.Bt.nnz);
+    if (c.divB) {
+      c.divB->v32 = f32_copy(c, c.divB->v64, 3 * (size_t)kDivS * L0.np);
+    } else {
+      c.B.v32 = f32_copy(c, c.B.v64, 3 * (size_t)c.B.nnz);
+      c.Bt.v32 = f32_copy(c, c.Bt.v64, 3 * (size_t)c.Bt.nnz);
+    }
     c.MQ.v32 = f32_copy(c, c.MQ.v64, c.MQ.nnz);
     c.LQ.v32 = f32_copy(c, c.LQ.v64, c.LQ.nnz);
     c.lumped_inv32 = f32_copy(c, c.lumped_inv64, L0.nvi);
@@ -383,10 +391,12 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
     c.symA->group = c.opt.spmv_group > 0 ? std::min(8, c.A.group) : 1;
     c.symA->batch = c.opt.sym_batch > 0 ? c.opt.sym_batch : 8;
   }
-  tune(c.B, 1, 2);
-  tune(c.Bt, 3, 3);
-  tune(c.B, 1, 2, 4);  // four right-hand sides (stokes_solve_multi)
-  tune(c.Bt, 3, 3, 4);
+  if (!c.divB) {
+    tune(c.B, 1, 2);
+    tune(c.Bt, 3, 3);
+    tune(c.B, 1, 2, 4);  // four right-hand sides (stokes_solve_multi)
+    tune(c.Bt, 3, 3, 4);
+  }
   tune(c.MQ, 1, 0);
   if (c.MV.v64) tune(c.MV, 3, 0);
   c.LQ.group = c.MQ.group;

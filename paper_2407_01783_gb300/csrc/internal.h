@@ -44,6 +44,19 @@ struct Error : std::runtime_error {
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// i / d for 0 <= i < 2^44 / d as a multiplication: with M = ceil(2^44 / d) the
+// product exceeds i 2^44 / d by less than i < 2^44 / d. Node indices (i < m^3,
+// d = m^2) satisfy it up to m = 445 points per axis, beyond the sizes whose
+// matrices fit 32-bit indices.
+struct FastDiv {
+  unsigned long long M;
+  int d;
+  explicit FastDiv(int d_) : M(((1ull << 44) + d_ - 1) / d_), d(d_) {}
+#ifdef __CUDACC__
+  __device__ __forceinline__ int div(int i) const { return (int)((i * M) >> 44); }
+#endif
+};
+
 // An NVTX range for the lifetime of the object (solver phases show up as
 // named ranges under a profiler; without one attached the calls do nothing).
 struct NvtxRange {
@@ -278,6 +291,18 @@ template <> inline float* Sym3Op::v<float>() const { return v32; }
 // br*bc planes of nnz entries each (plane j at v + j*nnz) so that consecutive
 // lanes read consecutive addresses.
 // ---------------------------------------------------------------------------
+// B in stencil storage (divergence.cu): block (1x3) of vertex k and the node at
+// half-grid offset e, value q at (3 e + q) np + k; serves B and B^T.
+constexpr int kDivS = 65;  // nodes that share a tetrahedron with a vertex
+struct DivOp {
+  int n = 0;
+  double* v64 = nullptr;
+  float* v32 = nullptr;
+  template <class T> T* v() const;
+};
+template <> inline double* DivOp::v<double>() const { return v64; }
+template <> inline float* DivOp::v<float>() const { return v32; }
+
 // The strain-form A of one level evaluated element by element in FP32
 // (element.cu): per-tetrahedron geometry and the work space of one product.
 constexpr int kElWords = 12;  // geometry words per tetrahedron
@@ -307,6 +332,7 @@ struct Csr {
                                   // double-float residual, and for all products if sym_products
   bool sym_products = false;
   const ElementOp* el = nullptr;  // FP32 products element by element instead (with sym_products)
+  const DivOp* div = nullptr;     // B and B^T: products from the stencil storage of B
   template <class T> T* v() const;
   double bytes(int elem) const {  // algorithmic bytes of one product (matrix only)
     return (double)nnz * (4.0 + elem * br * bc) + 4.0 * (rows + 1);
@@ -488,6 +514,14 @@ StencilOp* stencil_from_csr(const Exec& ex, Arena& ar, const StencilTables* st, 
 // Symmetric stencil storage of the BSR3 interior-P2 matrix m of level size n
 // (FP64 values; FP32 copies are made by the caller).
 Sym3Op* sym3_from_csr(const Exec& ex, Arena& ar, const StencilTables* st, int n, const Csr& m);
+// Stencil storage of B (FP64 values) from its CSR form, and the products
+// y = b + alpha B x, y = b + alpha s o (B^T x) for k = 1 or 4 right-hand sides
+DivOp* div_from_csr(const Exec& ex, Arena& ar, const StencilTables* st, int n, const Csr& B);
+void div_offsets(const StencilTables* st, signed char (*d)[3]);
+template <class T>
+void div_apply(const Exec& ex, const DivOp& d, int k, const T* x, T* y, const T* b, double alpha);
+template <class T>
+void divt_apply(const Exec& ex, const DivOp& d, int k, const T* x, T* y, const T* scale, const T* b, double alpha);
 void to_f32(const Exec& ex, const double* src, float* dst, size_t n);
 // lo = FP32(src - hi): with hi = FP32(src), hi + lo carries src to ~2^-48
 void to_f32_lo(const Exec& ex, const double* src, const float* hi, float* lo, size_t n);
@@ -831,6 +865,7 @@ struct stokes_ctx {
   // last forward solution (reduced) for the adjoint
   std::vector<std::unique_ptr<sk::StencilOp>> stencils;  // owned stencil storages
   std::unique_ptr<sk::Sym3Op> symA;                       // A in symmetric stencil storage
+  std::unique_ptr<sk::DivOp> divB;                        // B in stencil storage
   std::unique_ptr<sk::ElementOp> elA;                     // A element by element (mixed precision)
   double* U_last = nullptr;
   double* P_last = nullptr;

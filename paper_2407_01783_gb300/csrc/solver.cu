@@ -2026,6 +2026,18 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       convert<float, double>(c.ex, nv, yf, y);
       break;
     }
+    case STOKES_OP_B_F32:
+    case STOKES_OP_BT_F32: {
+      SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 B needs a mixed-precision context");
+      const bool div = op == STOKES_OP_B_F32;
+      const size_t nx = div ? nv : np, ny = div ? np : nv;
+      Tmp<float> xf(c.pool, nx), yf(c.pool, ny);
+      convert<double, float>(c.ex, nx, x, xf);
+      if (div) b_apply<float>(c.ex, c.B, xf, yf, (const float*)nullptr, 1.0);
+      else bt_apply<float>(c.ex, c.Bt, xf, yf, (const float*)nullptr, (const float*)nullptr, 1.0);
+      convert<float, double>(c.ex, ny, yf, y);
+      break;
+    }
     default: throw Error(STOKES_ERR_ARG, "unknown operator");
   }
   (void)np;

@@ -1123,6 +1123,11 @@ void bsr3_apply_dot_k(const Exec& ex, const Csr& m, int k, const T* x, T* y, con
 
 template <class T> void b_apply(const Exec& ex, const Csr& m, const T* x, T* y, const T* b, double alpha, int k) {
   SK_REQUIRE(k == 1 || k == 4, STOKES_ERR_ARG, "B product: 1 or 4 right-hand sides");
+  if (m.div) {  // the stored values once (its zero blocks not counted)
+    ProfScope ps(ex, STOKES_KERNEL_B, sizeof(T) * (3.0 * m.nnz + k * (3.0 * m.cols + m.rows * (b ? 2.0 : 1.0))));
+    div_apply<T>(ex, *m.div, k, x, y, b, alpha);
+    return;
+  }
   ProfScope ps(ex, STOKES_KERNEL_B, m.bytes(sizeof(T)) + sizeof(T) * k * (3.0 * m.cols + m.rows * (b ? 2.0 : 1.0)));
   if (k == 4) launch(ex, m, SH_B, x, EpiAxpy<T, 4>{b, nullptr, y, (T)alpha, (size_t)m.rows}, m.group4 ? m.group4 : m.group);
   else launch(ex, m, SH_B, x, EpiAxpy<T, 1>{b, nullptr, y, (T)alpha, (size_t)m.rows}, m.group);
@@ -1130,6 +1135,12 @@ template <class T> void b_apply(const Exec& ex, const Csr& m, const T* x, T* y, 
 template <class T> void bt_apply(const Exec& ex, const Csr& m, const T* x, T* y, const T* scale, const T* b,
                                  double alpha, int k) {
   SK_REQUIRE(k == 1 || k == 4, STOKES_ERR_ARG, "B^T product: 1 or 4 right-hand sides");
+  if (m.div) {
+    ProfScope ps(ex, STOKES_KERNEL_BT, sizeof(T) * (3.0 * m.nnz + k * (1.0 * m.cols + 3.0 * m.rows * (b ? 2.0 : 1.0)) +
+                                                    (scale ? m.rows : 0)));
+    divt_apply<T>(ex, *m.div, k, x, y, scale, b, alpha);
+    return;
+  }
   ProfScope ps(ex, STOKES_KERNEL_BT,
                m.bytes(sizeof(T)) +
                    sizeof(T) * (k * (1.0 * m.cols + 3.0 * m.rows * (b ? 2.0 : 1.0)) + (scale ? m.rows : 0)));

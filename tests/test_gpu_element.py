@@ -34,3 +34,23 @@ def test_fp32_strain_product(n, mu, dt):
     again = aos(host(S.apply("A_F32", cuda(soa(x)), x.size)))
     assert np.array_equal(y, again)
     S.close()
+
+
+@pytest.mark.parametrize("n", [2, 3, 5, 9, 14])
+def test_divergence_stencil(n):
+    """B and B^T from the shared stencil storage (n = 2, 3: offsets that alias
+    in the linear index; 14: several blocks per parity class), both precisions.
+    A row sums at most 65 x 3 products; FP64 alike to 1e-13."""
+    sk = gpu_module()
+    V = wl.kuhn_vertices(n, 0.16, 3)
+    S = sk.Stokes(n, V, 1e-2, 1e-3, 0.0, sk.stokes_default_options(precision=1))
+    orc = StokesSystem(KuhnMesh(n, V), 1e-2, 1e-3)
+    rng = np.random.default_rng(n)
+    u = rng.standard_normal(orc.B.shape[1]).astype(np.float32).astype(np.float64)
+    q = rng.standard_normal(orc.B.shape[0]).astype(np.float32).astype(np.float64)
+    for suffix, bound in (("", 1e-13), ("_F32", BOUND)):
+        bu = host(S.apply("B" + suffix, cuda(soa(u)), q.size))
+        btq = aos(host(S.apply("BT" + suffix, cuda(q), u.size)))
+        assert np.linalg.norm(bu - orc.B @ u) <= bound * np.linalg.norm(abs(orc.B) @ abs(u))
+        assert np.linalg.norm(btq - orc.B.T @ q) <= bound * np.linalg.norm(abs(orc.B.T) @ abs(q))
+    S.close()
