@@ -283,6 +283,8 @@ typedef enum {
                                  only)                                        */
   STOKES_OP_B_F32 = 20,       /* y = B x, likewise                            */
   STOKES_OP_BT_F32 = 21,      /* y = B^T x, likewise                          */
+  STOKES_OP_PROLONG_P2_F32 = 22,  /* as PROLONG_P2 in FP32, likewise        */
+  STOKES_OP_RESTRICT_P2_F32 = 23, /* as RESTRICT_P2 in FP32, likewise       */
   STOKES_OP_VCYCLE_VEL = 18   /* y = the configured velocity preconditioner
                                  (vcycles V-cycles of A~_{vel_prec}) applied
                                  to x, from level 0                          */

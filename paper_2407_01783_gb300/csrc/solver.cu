@@ -396,6 +396,22 @@ template <class T> static bool use_split(const stokes_ctx& c, int which, bool il
   return wanted && which == 0 && c.lv.size() >= 2 && c.lv[0].A3.st != nullptr && stencil_in_use<T>(c.lv[0].A3, il);
 }
 
+// FP32 P2 transfers between levels l and l + 1 (transfer.cu): without matrices
+// unless the caller asked for CSR everywhere; restriction on nested levels only
+static bool implicit_transfers(const stokes_ctx& c) { return c.opt.format != 1; }
+static double transfer_bytes(const stokes_ctx& c, int l, int nr, int fine_streams) {
+  return 4.0 * nr * ((double)c.lv[l].nvi * fine_streams + c.lv[l + 1].nvi);
+}
+static bool restrict_p2_level(stokes_ctx& c, int l, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
+  if (c.lv[l].n != 2 * c.lv[l + 1].n) return false;
+  ProfScope ps(c.ex, STOKES_KERNEL_TRANSFER, transfer_bytes(c, l, nr, 1));
+  return restrict_p2(c.ex, c.lv[l].n, c.lv[l + 1].n, nr, x, y, il, sm);
+}
+static void prolong_p2_level(stokes_ctx& c, int l, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
+  ProfScope ps(c.ex, STOKES_KERNEL_TRANSFER, transfer_bytes(c, l, nr, 2));
+  prolong_p2(c.ex, c.lv[l].n, c.lv[l + 1].n, nr, x, y, il, sm);
+}
+
 // il: node-interleaved level vectors (K > 1); split: level 0 parity-split
 // numbered (b, x and the temporaries of level 0)
 template <class T>
@@ -430,10 +446,17 @@ static void vcycle(stokes_ctx& c, int which, int l, const T* b, T* x, bool xzero
   size_t lenc = (size_t)Mc.rows * nr;
   // transfers from / to this level (the coarse level is always natural)
   auto restrict_to = [&](const T* r, T* bc) {
+    if constexpr (std::is_same<T, float>::value)
+      if (which != 1 && implicit_transfers(c) && restrict_p2_level(c, l, nr, r, bc, il, split ? &sm : nullptr)) return;
     if (split) restrict_split<T>(c.ex, L.R2, nr, r, bc, il, sm);
     else spmv_store<T>(c.ex, which == 1 ? L.R1 : L.R2, nr, r, bc, STOKES_KERNEL_TRANSFER, il);
   };
   auto prolong_into = [&](const T* xc, T* xf) {
+    if constexpr (std::is_same<T, float>::value)
+      if (which != 1 && implicit_transfers(c)) {
+        prolong_p2_level(c, l, nr, xc, xf, il, split ? &sm : nullptr);
+        return;
+      }
     if (split) prolong_add_split<T>(c.ex, L.P2, nr, xc, xf, il, sm);
     else spmv_add<T>(c.ex, which == 1 ? L.P1 : L.P2, nr, xc, xf, STOKES_KERNEL_TRANSFER, il);
   };
@@ -1955,7 +1978,7 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
   stokes_ctx& c = *cp;
   SK_REQUIRE(level >= 0 && level < (int)c.lv.size(), STOKES_ERR_ARG, "level out of range");
   const Level& L = c.lv[level];
-  if (op != STOKES_OP_A3 && op != STOKES_OP_KQ && op != STOKES_OP_VCYCLE_A3 && op != STOKES_OP_PROLONG_P2 &&
+  if (op != STOKES_OP_PROLONG_P2_F32 && op != STOKES_OP_RESTRICT_P2_F32 && op != STOKES_OP_A3 && op != STOKES_OP_KQ && op != STOKES_OP_VCYCLE_A3 && op != STOKES_OP_PROLONG_P2 &&
       op != STOKES_OP_RESTRICT_P2 && op != STOKES_OP_PROLONG_P1)
     SK_REQUIRE(level == 0, STOKES_ERR_ARG, "operator defined on level 0 only");
   const size_t np = npres(c), nv = nvel(c);
@@ -2036,6 +2059,25 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       if (div) b_apply<float>(c.ex, c.B, xf, yf, (const float*)nullptr, 1.0);
       else bt_apply<float>(c.ex, c.Bt, xf, yf, (const float*)nullptr, (const float*)nullptr, 1.0);
       convert<float, double>(c.ex, ny, yf, y);
+      break;
+    }
+    case STOKES_OP_PROLONG_P2_F32:
+    case STOKES_OP_RESTRICT_P2_F32: {
+      SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 transfers need a mixed-precision context");
+      SK_REQUIRE(level + 1 < (int)c.lv.size(), STOKES_ERR_ARG, "no coarser level");
+      const bool up = op == STOKES_OP_PROLONG_P2_F32;
+      const size_t nf = 3 * (size_t)L.nvi, nco = 3 * (size_t)c.lv[level + 1].nvi;
+      Tmp<float> xf(c.pool, up ? nco : nf), yf(c.pool, up ? nf : nco);
+      convert<double, float>(c.ex, up ? nco : nf, x, xf);
+      const float* xs = xf;
+      if (up) {
+        zero<float>(c, yf, nf);
+        if (implicit_transfers(c)) prolong_p2_level(c, level, 3, xs, yf, false, nullptr);
+        else spmv_add<float>(c.ex, L.P2, 3, xs, yf, STOKES_KERNEL_TRANSFER);
+      } else if (!implicit_transfers(c) || !restrict_p2_level(c, level, 3, xs, yf, false, nullptr)) {
+        spmv_store<float>(c.ex, L.R2, 3, xs, yf, STOKES_KERNEL_TRANSFER);
+      }
+      convert<float, double>(c.ex, up ? nf : nco, yf, y);
       break;
     }
     default: throw Error(STOKES_ERR_ARG, "unknown operator");

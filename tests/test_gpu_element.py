@@ -54,3 +54,26 @@ def test_divergence_stencil(n):
         assert np.linalg.norm(bu - orc.B @ u) <= bound * np.linalg.norm(abs(orc.B) @ abs(u))
         assert np.linalg.norm(btq - orc.B.T @ q) <= bound * np.linalg.norm(abs(orc.B.T) @ abs(q))
     S.close()
+
+
+@pytest.mark.parametrize("n", [4, 5, 7, 8, 12, 33])
+def test_fp32_transfers_without_matrices(n):
+    """Prolongation (nested and odd meshes) and restriction (nested) in FP32
+    against the assembled FP64 transfer matrices, on every level."""
+    sk = gpu_module()
+    S = sk.Stokes(n, wl.kuhn_vertices(n, 0.1, 1), 1e-2, 1e-3, 0.0, sk.stokes_default_options(precision=1))
+    rng = np.random.default_rng(n)
+    sizes, m = [], n
+    while True:
+        sizes.append(3 * (2 * m - 1) ** 3)
+        if m < 4:
+            break
+        m = (m + 1) // 2
+    for level in range(len(sizes) - 1):
+        for op, nx, ny in (("PROLONG_P2", sizes[level + 1], sizes[level]), ("RESTRICT_P2", sizes[level], sizes[level + 1])):
+            x = rng.standard_normal(nx).astype(np.float32).astype(np.float64)
+            want = host(S.apply(op, cuda(x), ny, level))
+            size = host(S.apply(op, cuda(abs(x)), ny, level))  # (weights of both signs: a lower bound of |P||x|)
+            got = host(S.apply(op + "_F32", cuda(x), ny, level))
+            assert np.linalg.norm(got - want) <= BOUND * (np.linalg.norm(size) + np.linalg.norm(want))
+    S.close()
