@@ -44,6 +44,7 @@ template <class T> struct DotArgs {
 
 template <class T, int K>
 __global__ void __launch_bounds__(256) k_dots(DotArgs<T> a) {
+  dep_wait();
   double s[K];
 #pragma unroll
   for (int j = 0; j < K; ++j) s[j] = 0.0;
@@ -162,10 +163,10 @@ void dots(const Exec& ex, const DotScratch& ds, int k, const T* const* x, const 
   a.out = out;
   int grid = (int)std::min<long long>(kDotBlocks, std::max<long long>(1, cdiv((long long)n, 256)));
   switch (k) {
-    case 1: k_dots<T, 1><<<grid, 256, 0, ex.s>>>(a); break;
-    case 2: k_dots<T, 2><<<grid, 256, 0, ex.s>>>(a); break;
-    case 3: k_dots<T, 3><<<grid, 256, 0, ex.s>>>(a); break;
-    default: k_dots<T, 4><<<grid, 256, 0, ex.s>>>(a); break;
+    case 1: launch_dep(k_dots<T, 1>, grid, 256, 0, ex, a); break;
+    case 2: launch_dep(k_dots<T, 2>, grid, 256, 0, ex, a); break;
+    case 3: launch_dep(k_dots<T, 3>, grid, 256, 0, ex, a); break;
+    default: launch_dep(k_dots<T, 4>, grid, 256, 0, ex, a); break;
   }
   SK_CHECK_LAUNCH();
 }
@@ -193,6 +194,7 @@ template <class T> struct MultiArgs {
 // accumulators are indexed statically
 template <class T, int K>
 __global__ void __launch_bounds__(256) k_mdot(MultiArgs<T> a) {
+  dep_wait();
   double s[K];
   if constexpr (std::is_same<T, float>::value) {
     // FP32 vectors: per-thread double-float sums (df_dot) on the FP32 units
@@ -252,6 +254,7 @@ __global__ void __launch_bounds__(256) k_mdot(MultiArgs<T> a) {
 
 template <class T, int K>
 __global__ void __launch_bounds__(256) k_maxpy(MultiArgs<T> a) {
+  dep_wait();
   __shared__ T h[K];
   if (threadIdx.x < K) h[threadIdx.x] = threadIdx.x < a.k ? (T)(a.sign * (a.dev ? a.dev[threadIdx.x] : a.c[threadIdx.x])) : T(0);
   __syncthreads();
@@ -285,12 +288,12 @@ void mdot(const Exec& ex, const DotScratch& ds, int k, const T* const* V, const 
   a.counter = ds.fused_counter;
   a.out = out;
   switch (pow2_at_least(k)) {
-    case 1: k_mdot<T, 1><<<grid, 256, 0, ex.s>>>(a); break;
-    case 2: k_mdot<T, 2><<<grid, 256, 0, ex.s>>>(a); break;
-    case 4: k_mdot<T, 4><<<grid, 256, 0, ex.s>>>(a); break;
-    case 8: k_mdot<T, 8><<<grid, 256, 0, ex.s>>>(a); break;
-    case 16: k_mdot<T, 16><<<grid, 256, 0, ex.s>>>(a); break;
-    default: k_mdot<T, 32><<<grid, 256, 0, ex.s>>>(a); break;
+    case 1: launch_dep(k_mdot<T, 1>, grid, 256, 0, ex, a); break;
+    case 2: launch_dep(k_mdot<T, 2>, grid, 256, 0, ex, a); break;
+    case 4: launch_dep(k_mdot<T, 4>, grid, 256, 0, ex, a); break;
+    case 8: launch_dep(k_mdot<T, 8>, grid, 256, 0, ex, a); break;
+    case 16: launch_dep(k_mdot<T, 16>, grid, 256, 0, ex, a); break;
+    default: launch_dep(k_mdot<T, 32>, grid, 256, 0, ex, a); break;
   }
   SK_CHECK_LAUNCH();
 }
@@ -313,12 +316,12 @@ void maxpy(const Exec& ex, int k, const double* dev_coef, const double* host_coe
   a.w = w;
   const int grid = (int)std::min<long long>(cdiv((long long)n, 256), 8 * 152);  // as the elementwise kernels
   switch (pow2_at_least(k)) {
-    case 1: k_maxpy<T, 1><<<grid, 256, 0, ex.s>>>(a); break;
-    case 2: k_maxpy<T, 2><<<grid, 256, 0, ex.s>>>(a); break;
-    case 4: k_maxpy<T, 4><<<grid, 256, 0, ex.s>>>(a); break;
-    case 8: k_maxpy<T, 8><<<grid, 256, 0, ex.s>>>(a); break;
-    case 16: k_maxpy<T, 16><<<grid, 256, 0, ex.s>>>(a); break;
-    default: k_maxpy<T, 32><<<grid, 256, 0, ex.s>>>(a); break;
+    case 1: launch_dep(k_maxpy<T, 1>, grid, 256, 0, ex, a); break;
+    case 2: launch_dep(k_maxpy<T, 2>, grid, 256, 0, ex, a); break;
+    case 4: launch_dep(k_maxpy<T, 4>, grid, 256, 0, ex, a); break;
+    case 8: launch_dep(k_maxpy<T, 8>, grid, 256, 0, ex, a); break;
+    case 16: launch_dep(k_maxpy<T, 16>, grid, 256, 0, ex, a); break;
+    default: launch_dep(k_maxpy<T, 32>, grid, 256, 0, ex, a); break;
   }
   SK_CHECK_LAUNCH();
 }
@@ -328,7 +331,7 @@ void maxpy(const Exec& ex, int k, const double* dev_coef, const double* host_coe
 // once per ~8 elements per thread rather than once per 256 elements.
 constexpr int kEwBlocks = 8 * 152;
 static inline int ew_grid(size_t n) { return (int)std::min<long long>(cdiv((long long)n, 256), kEwBlocks); }
-#define SK_GRID(n) ew_grid(n), 256, 0, ex.s
+#define SK_GRID(n) ew_grid(n), 256, 0, ex
 #define SK_LOOP(i) \
   _Pragma("unroll 4") for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
 
@@ -345,6 +348,7 @@ static inline int ew_grid(size_t n) { return (int)std::min<long long>(cdiv((long
 
 template <class T>
 __global__ void k_axpby(size_t n, Coef a, const T* __restrict__ x, Coef b, T* __restrict__ y, int* flag) {
+  dep_wait();
   SK_COEF2(a, b, ad, bd);
   const T av = (T)ad, bv = (T)bd;
   if (bv == T(0)) {
@@ -356,13 +360,14 @@ __global__ void k_axpby(size_t n, Coef a, const T* __restrict__ x, Coef b, T* __
 template <class T> void axpby(const Exec& ex, size_t n, Coef a, const T* x, Coef b, T* y) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 3);
-  k_axpby<T><<<SK_GRID(n)>>>(n, a, x, b, y, ex.flag);
+  launch_dep(k_axpby<T>, SK_GRID(n), n, a, x, b, y, ex.flag);
   SK_CHECK_LAUNCH();
 }
 
 template <class T>
 __global__ void k_cg_update(size_t n, Coef a, const T* __restrict__ d, T* __restrict__ x, const T* __restrict__ q,
                             T* __restrict__ r, int* flag) {
+  dep_wait();
   SK_COEF2(a, a, ad, unused);
   (void)unused;
   if (blockIdx.x == 0 && threadIdx.x == 0 && flag && a.den && !(*a.den > 0.0))
@@ -380,7 +385,7 @@ __global__ void k_cg_update(size_t n, Coef a, const T* __restrict__ d, T* __rest
 template <class T> void cg_update(const Exec& ex, size_t n, Coef a, const T* d, T* x, const T* q, T* r) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * (r ? 6 : 3));
-  k_cg_update<T><<<SK_GRID(n)>>>(n, a, d, x, q, r, ex.flag);
+  launch_dep(k_cg_update<T>, SK_GRID(n), n, a, d, x, q, r, ex.flag);
   SK_CHECK_LAUNCH();
 }
 
@@ -389,6 +394,7 @@ template <class T> void cg_update(const Exec& ex, size_t n, Coef a, const T* d, 
 template <class T>
 __global__ void k_cg_update_rr(size_t n, Coef a, const T* __restrict__ d, T* __restrict__ x, const T* __restrict__ q,
                                T* __restrict__ r, int* flag, double* partial, unsigned* counter, double* rr) {
+  dep_wait();
   SK_COEF2(a, a, ad, unused);
   (void)unused;
   if (blockIdx.x == 0 && threadIdx.x == 0 && flag && a.den && !(*a.den > 0.0))
@@ -410,12 +416,13 @@ void cg_update_rr(const Exec& ex, const DotScratch& ds, size_t n, Coef a, const 
   const int grid = ew_grid(n);
   SK_REQUIRE(ds.fused_partial && grid <= ds.fused_cap, STOKES_ERR_ARG, "fused dot scratch too small");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 6);
-  k_cg_update_rr<T><<<grid, 256, 0, ex.s>>>(n, a, d, x, q, r, ex.flag, ds.fused_partial, ds.fused_counter, rr);
+  launch_dep(k_cg_update_rr<T>, grid, 256, 0, ex, n, a, d, x, q, r, ex.flag, ds.fused_partial, ds.fused_counter, rr);
   SK_CHECK_LAUNCH();
 }
 
 template <class T>
 __global__ void k_scale_copy(size_t n, Coef a, const T* __restrict__ x, T* __restrict__ y, int* flag) {
+  dep_wait();
   SK_COEF2(a, a, ad, unused);
   (void)unused;
   SK_LOOP(i) {
@@ -425,12 +432,13 @@ __global__ void k_scale_copy(size_t n, Coef a, const T* __restrict__ x, T* __res
 template <class T> void scale_copy(const Exec& ex, size_t n, Coef a, const T* x, T* y) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 2);
-  k_scale_copy<T><<<SK_GRID(n)>>>(n, a, x, y, ex.flag);
+  launch_dep(k_scale_copy<T>, SK_GRID(n), n, a, x, y, ex.flag);
   SK_CHECK_LAUNCH();
 }
 
 template <class T>
 __global__ void k_lincomb2(size_t n, T c1, const T* __restrict__ x1, T c2, const T* __restrict__ x2, T* __restrict__ y) {
+  dep_wait();
   SK_LOOP(i) {
     y[i] = c1 * x1[i] + c2 * x2[i];
   }
@@ -438,11 +446,12 @@ __global__ void k_lincomb2(size_t n, T c1, const T* __restrict__ x1, T c2, const
 template <class T> void lincomb2(const Exec& ex, size_t n, double c1, const T* x1, double c2, const T* x2, T* y) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 3);
-  k_lincomb2<T><<<SK_GRID(n)>>>(n, (T)c1, x1, (T)c2, x2, y);
+  launch_dep(k_lincomb2<T>, SK_GRID(n), n, (T)c1, x1, (T)c2, x2, y);
   SK_CHECK_LAUNCH();
 }
 
 template <class T> __global__ void k_sub_ratio(size_t n, const double* num, const double* den, double scale, T* x) {
+  dep_wait();
   __shared__ double sk_v;
   if (threadIdx.x == 0) sk_v = scale * (*num) / (den ? *den : 1.0);
   __syncthreads();
@@ -453,19 +462,20 @@ template <class T> __global__ void k_sub_ratio(size_t n, const double* num, cons
 template <class T> void sub_mean(const Exec& ex, size_t n, const double* sum, double count, T* r) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 2);
-  k_sub_ratio<T><<<SK_GRID(n)>>>(n, sum, nullptr, 1.0 / count, r);
+  launch_dep(k_sub_ratio<T>, SK_GRID(n), n, sum, nullptr, 1.0 / count, r);
   SK_CHECK_LAUNCH();
 }
 template <class T> void sub_ratio(const Exec& ex, size_t n, const double* num, const double* den, T* x) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * 2);
-  k_sub_ratio<T><<<SK_GRID(n)>>>(n, num, den, 1.0, x);
+  launch_dep(k_sub_ratio<T>, SK_GRID(n), n, num, den, 1.0, x);
   SK_CHECK_LAUNCH();
 }
 
 template <class T>
 __global__ void k_cheb_first(size_t n, const T* __restrict__ dinv, const T* __restrict__ b, T c,
                              T* __restrict__ d, T* __restrict__ x) {
+  dep_wait();
   // component-major: blockIdx.y is the component, n the rows of one component
   const size_t off = (size_t)blockIdx.y * n;
   SK_LOOP(i) {
@@ -478,7 +488,7 @@ template <class T> void cheb_first(const Exec& ex, size_t n, int nr, const T* di
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * (n * 3 + n / nr));
   const size_t rows = n / nr;
-  k_cheb_first<T><<<dim3(std::max(1, ew_grid(rows) / nr), nr), 256, 0, ex.s>>>(rows, dinv, b, (T)c, d, x);
+  launch_dep(k_cheb_first<T>, dim3(std::max(1, ew_grid(rows) / nr), nr), 256, 0, ex, rows, dinv, b, (T)c, d, x);
   SK_CHECK_LAUNCH();
 }
 
@@ -486,6 +496,7 @@ template <class T> void cheb_first(const Exec& ex, size_t n, int nr, const T* di
 template <class T, int NR>
 __global__ void k_cheb_first_il(size_t n, const T* __restrict__ dinv, const T* __restrict__ b, T c,
                                 T* __restrict__ d, T* __restrict__ x) {
+  dep_wait();
   SK_LOOP(i) {
     const T s = c * dinv[i];
 #pragma unroll
@@ -502,8 +513,8 @@ void cheb_first_il(const Exec& ex, size_t n, int nr, const T* dinv, const T* b, 
   SK_REQUIRE(nr == 4 || nr == 12, STOKES_ERR_ARG, "interleaved vectors need 4 or 12 components");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * (n * 3 + n / nr));
   const size_t rows = n / nr;
-  if (nr == 4) k_cheb_first_il<T, 4><<<SK_GRID(rows)>>>(rows, dinv, b, (T)c, d, x);
-  else k_cheb_first_il<T, 12><<<SK_GRID(rows)>>>(rows, dinv, b, (T)c, d, x);
+  if (nr == 4) launch_dep(k_cheb_first_il<T, 4>, SK_GRID(rows), rows, dinv, b, (T)c, d, x);
+  else launch_dep(k_cheb_first_il<T, 12>, SK_GRID(rows), rows, dinv, b, (T)c, d, x);
   SK_CHECK_LAUNCH();
 }
 
@@ -511,6 +522,7 @@ void cheb_first_il(const Exec& ex, size_t n, int nr, const T* dinv, const T* b, 
 // read coalesced across the warp) and writes them contiguously, or back
 template <class T, int NR, bool TO_IL>
 __global__ void k_relayout(size_t n, const T* __restrict__ src, T* __restrict__ dst) {
+  dep_wait();
   // n rows
   SK_LOOP(i) {
 #pragma unroll
@@ -524,16 +536,16 @@ template <class T> void to_interleaved(const Exec& ex, size_t rows, int nr, cons
   if (!rows) return;
   SK_REQUIRE(nr == 4 || nr == 12, STOKES_ERR_ARG, "interleaved vectors need 4 or 12 components");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, 2.0 * sizeof(T) * rows * nr);
-  if (nr == 4) k_relayout<T, 4, true><<<SK_GRID(rows)>>>(rows, cm, il);
-  else k_relayout<T, 12, true><<<SK_GRID(rows)>>>(rows, cm, il);
+  if (nr == 4) launch_dep(k_relayout<T, 4, true>, SK_GRID(rows), rows, cm, il);
+  else launch_dep(k_relayout<T, 12, true>, SK_GRID(rows), rows, cm, il);
   SK_CHECK_LAUNCH();
 }
 template <class T> void to_component_major(const Exec& ex, size_t rows, int nr, const T* il, T* cm) {
   if (!rows) return;
   SK_REQUIRE(nr == 4 || nr == 12, STOKES_ERR_ARG, "interleaved vectors need 4 or 12 components");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, 2.0 * sizeof(T) * rows * nr);
-  if (nr == 4) k_relayout<T, 4, false><<<SK_GRID(rows)>>>(rows, il, cm);
-  else k_relayout<T, 12, false><<<SK_GRID(rows)>>>(rows, il, cm);
+  if (nr == 4) launch_dep(k_relayout<T, 4, false>, SK_GRID(rows), rows, il, cm);
+  else launch_dep(k_relayout<T, 12, false>, SK_GRID(rows), rows, il, cm);
   SK_CHECK_LAUNCH();
 }
 
@@ -542,6 +554,7 @@ template <class T> void to_component_major(const Exec& ex, size_t rows, int nr, 
 // [rows][nr]; a thread per natural row i
 template <class T, int NR, bool IL, bool TO>
 __global__ void k_split(size_t n, SplitMap sm, const T* __restrict__ src, T* __restrict__ dst) {
+  dep_wait();
   SK_LOOP(i) {
     const size_t j = (size_t)sm((int)i);
 #pragma unroll
@@ -559,12 +572,12 @@ static void split_launch(const Exec& ex, size_t rows, int nr, const T* src, T* d
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, 2.0 * sizeof(T) * rows * nr);
   if (il) {
     SK_REQUIRE(nr == 4 || nr == 12, STOKES_ERR_ARG, "interleaved vectors need 4 or 12 components");
-    if (nr == 4) k_split<T, 4, true, TO><<<SK_GRID(rows)>>>(rows, sm, src, dst);
-    else k_split<T, 12, true, TO><<<SK_GRID(rows)>>>(rows, sm, src, dst);
+    if (nr == 4) launch_dep(k_split<T, 4, true, TO>, SK_GRID(rows), rows, sm, src, dst);
+    else launch_dep(k_split<T, 12, true, TO>, SK_GRID(rows), rows, sm, src, dst);
   } else {
     SK_REQUIRE(nr == 1 || nr == 3, STOKES_ERR_ARG, "split numbering: 1 or 3 components (component-major)");
-    if (nr == 1) k_split<T, 1, false, TO><<<SK_GRID(rows)>>>(rows, sm, src, dst);
-    else k_split<T, 3, false, TO><<<SK_GRID(rows)>>>(rows, sm, src, dst);
+    if (nr == 1) launch_dep(k_split<T, 1, false, TO>, SK_GRID(rows), rows, sm, src, dst);
+    else launch_dep(k_split<T, 3, false, TO>, SK_GRID(rows), rows, sm, src, dst);
   }
   SK_CHECK_LAUNCH();
 }
@@ -577,6 +590,7 @@ void from_split(const Exec& ex, size_t rows, int nr, const T* src, T* dst, bool 
 }
 
 template <class S, class D> __global__ void k_convert(size_t n, const S* __restrict__ x, D* __restrict__ y) {
+  dep_wait();
   SK_LOOP(i) {
     y[i] = (D)x[i];
   }
@@ -584,10 +598,11 @@ template <class S, class D> __global__ void k_convert(size_t n, const S* __restr
 template <class S, class D> void convert(const Exec& ex, size_t n, const S* x, D* y) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + sizeof(D)) * n);
-  k_convert<S, D><<<SK_GRID(n)>>>(n, x, y);
+  launch_dep(k_convert<S, D>, SK_GRID(n), n, x, y);
   SK_CHECK_LAUNCH();
 }
 template <class S, class D> __global__ void k_add_convert(size_t n, const S* __restrict__ x, D* __restrict__ y) {
+  dep_wait();
   SK_LOOP(i) {
     y[i] += (D)x[i];
   }
@@ -595,12 +610,13 @@ template <class S, class D> __global__ void k_add_convert(size_t n, const S* __r
 template <class S, class D> void add_convert(const Exec& ex, size_t n, const S* x, D* y) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + 2 * sizeof(D)) * n);
-  k_add_convert<S, D><<<SK_GRID(n)>>>(n, x, y);
+  launch_dep(k_add_convert<S, D>, SK_GRID(n), n, x, y);
   SK_CHECK_LAUNCH();
 }
 
 // reduced interior velocity [(2n-1)^3][3] <-> all-node field [(2n+1)^3][3]
 __global__ void k_expand(int n, const double* __restrict__ ured, double* __restrict__ uall) {
+  dep_wait();
   int N = 2 * n + 1, m = 2 * n - 1;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t tot = (size_t)N * N * N;
@@ -614,10 +630,11 @@ __global__ void k_expand(int n, const double* __restrict__ ured, double* __restr
 void expand_velocity(const Exec& ex, int n, const double* ured, double* uall) {
   size_t tot = (size_t)(2 * n + 1) * (2 * n + 1) * (2 * n + 1);
   ProfScope ps(ex, STOKES_KERNEL_OTHER, 48.0 * tot);
-  k_expand<<<cdiv((long long)tot, 256), 256, 0, ex.s>>>(n, ured, uall);  // one thread per node
+  launch_dep(k_expand, cdiv((long long)tot, 256), 256, 0, ex, n, ured, uall);  // one thread per node
   SK_CHECK_LAUNCH();
 }
 __global__ void k_restrict_vel(int n, const double* __restrict__ uall, double* __restrict__ ured) {
+  dep_wait();
   int N = 2 * n + 1, m = 2 * n - 1;
   size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t tot = (size_t)m * m * m;
@@ -629,17 +646,19 @@ __global__ void k_restrict_vel(int n, const double* __restrict__ uall, double* _
 void restrict_velocity(const Exec& ex, int n, const double* uall, double* ured) {
   size_t tot = (size_t)(2 * n - 1) * (2 * n - 1) * (2 * n - 1);
   ProfScope ps(ex, STOKES_KERNEL_OTHER, 48.0 * tot);
-  k_restrict_vel<<<cdiv((long long)tot, 256), 256, 0, ex.s>>>(n, uall, ured);
+  launch_dep(k_restrict_vel, cdiv((long long)tot, 256), 256, 0, ex, n, uall, ured);
   SK_CHECK_LAUNCH();
 }
 
 __global__ void k_nonfinite(size_t n, const double* __restrict__ x, int* flag) {
+  dep_wait();
   SK_LOOP(i) {
     if (!isfinite(x[i])) atomicOr(flag, 2);
   }
 }
 __global__ void k_split_f64(size_t n, const double* __restrict__ x, float* __restrict__ hi,
                             float* __restrict__ lo) {
+  dep_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const double v = x[i];
     const float h = (float)v;
@@ -651,21 +670,21 @@ __global__ void k_split_f64(size_t n, const double* __restrict__ x, float* __res
 void split_f64(const Exec& ex, size_t n, const double* x, float* hi, float* lo) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, 16.0 * n);
-  k_split_f64<<<(unsigned)std::min<size_t>(cdiv(n, 256), 1 << 20), 256, 0, ex.s>>>(n, x, hi, lo);
+  launch_dep(k_split_f64, (unsigned)std::min<size_t>(cdiv(n, 256), 1 << 20), 256, 0, ex, n, x, hi, lo);
   SK_CHECK_LAUNCH();
 }
 
 void count_nonfinite(const Exec& ex, size_t n, const double* x, int* flag) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_OTHER, 8.0 * n);
-  k_nonfinite<<<SK_GRID(n)>>>(n, x, flag);
+  launch_dep(k_nonfinite, SK_GRID(n), n, x, flag);
   SK_CHECK_LAUNCH();
 }
 
-__global__ void k_scalar_sub(double* out, const double* a, const double* b) { *out = *a - *b; }
+__global__ void k_scalar_sub(double* out, const double* a, const double* b) { dep_wait(); *out = *a - *b; }
 void scalar_sub(const Exec& ex, double* out, const double* a, const double* b) {
   ProfScope ps(ex, STOKES_KERNEL_OTHER, 24.0);
-  k_scalar_sub<<<1, 1, 0, ex.s>>>(out, a, b);
+  launch_dep(k_scalar_sub, 1, 1, 0, ex, out, a, b);
   SK_CHECK_LAUNCH();
 }
 

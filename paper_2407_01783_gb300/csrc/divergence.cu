@@ -46,6 +46,7 @@ template <int E, int K> __device__ constexpr int div_d() {
 
 __global__ void k_div_fill(int n, DivOffsets t, const int* __restrict__ rp, const int* __restrict__ col, long long nnz,
                            const double* __restrict__ val, double* __restrict__ out) {
+  dep_wait();
   const int nv = n + 1, np = nv * nv * nv, m = 2 * n - 1;
   const int r = blockIdx.x * blockDim.x + threadIdx.x, e = blockIdx.y;
   if (r >= np) return;
@@ -75,7 +76,7 @@ DivOp* div_from_csr(const Exec& ex, Arena& ar, const StencilTables* st, int n, c
   o->n = n;
   const int np = (n + 1) * (n + 1) * (n + 1);
   o->v64 = ar.alloc<double>((size_t)3 * kDivS * np);
-  k_div_fill<<<dim3(cdiv(np, 256), kDivS), 256, 0, ex.s>>>(n, t, B.rowptr, B.col, B.nnz, B.v64, o->v64);
+  launch_dep(k_div_fill, dim3(cdiv(np, 256), kDivS), 256, 0, ex, n, t, B.rowptr, B.col, B.nnz, B.v64, o->v64);
   SK_CHECK_LAUNCH();
   return o;
 }
@@ -130,6 +131,7 @@ __device__ __forceinline__ void div_warp(int w, const T* __restrict__ v, const T
 template <int K, class T>
 __global__ void __launch_bounds__(256, 4) k_div(int n, FastDiv by_v, FastDiv by_vv, const T* __restrict__ v,
                                                 const T* __restrict__ x, const T* b, T alpha, T* y) {
+  dep_wait();
   __shared__ T sh[8][K][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nv = n + 1, np = nv * nv * nv, m = 2 * n - 1;
@@ -187,6 +189,7 @@ template <int K, class T>
 __global__ void __launch_bounds__(256) k_divt(int n, FastDiv by_o, FastDiv by_e, const T* __restrict__ v,
                                               const T* __restrict__ x, const T* __restrict__ scale, const T* b, T alpha,
                                               T* y) {
+  dep_wait();
   const int c = blockIdx.y, nv = n + 1, np = nv * nv * nv, m = 2 * n - 1;
   const int odd[3] = {c & 1, (c >> 1) & 1, c >> 2};
   const int ex = n - 1 + odd[0], ey = n - 1 + odd[1], ez = n - 1 + odd[2];
@@ -215,16 +218,16 @@ template <class T>
 void div_apply(const Exec& ex, const DivOp& d, int k, const T* x, T* y, const T* b, double alpha) {
   const int np = (d.n + 1) * (d.n + 1) * (d.n + 1);
   const FastDiv by_v(d.n + 1), by_vv((d.n + 1) * (d.n + 1));
-  if (k == 4) k_div<4, T><<<cdiv(np, 32), 256, 0, ex.s>>>(d.n, by_v, by_vv, d.template v<T>(), x, b, (T)alpha, y);
-  else k_div<1, T><<<cdiv(np, 32), 256, 0, ex.s>>>(d.n, by_v, by_vv, d.template v<T>(), x, b, (T)alpha, y);
+  if (k == 4) launch_dep(k_div<4, T>, cdiv(np, 32), 256, 0, ex, d.n, by_v, by_vv, d.template v<T>(), x, b, (T)alpha, y);
+  else launch_dep(k_div<1, T>, cdiv(np, 32), 256, 0, ex, d.n, by_v, by_vv, d.template v<T>(), x, b, (T)alpha, y);
   SK_CHECK_LAUNCH();
 }
 template <class T>
 void divt_apply(const Exec& ex, const DivOp& d, int k, const T* x, T* y, const T* scale, const T* b, double alpha) {
   const dim3 grid(cdiv((long long)d.n * d.n * d.n, 256), 8);
   const FastDiv by_o(d.n), by_e(d.n - 1);
-  if (k == 4) k_divt<4, T><<<grid, 256, 0, ex.s>>>(d.n, by_o, by_e, d.template v<T>(), x, scale, b, (T)alpha, y);
-  else k_divt<1, T><<<grid, 256, 0, ex.s>>>(d.n, by_o, by_e, d.template v<T>(), x, scale, b, (T)alpha, y);
+  if (k == 4) launch_dep(k_divt<4, T>, grid, 256, 0, ex, d.n, by_o, by_e, d.template v<T>(), x, scale, b, (T)alpha, y);
+  else launch_dep(k_divt<1, T>, grid, 256, 0, ex, d.n, by_o, by_e, d.template v<T>(), x, scale, b, (T)alpha, y);
   SK_CHECK_LAUNCH();
 }
 

@@ -55,6 +55,7 @@ __host__ __device__ constexpr int el_node(int p, int a) {
 // them as three coalesced 16-byte loads per lane.
 __host__ __device__ __forceinline__ size_t el_blocks(size_t nc) { return (nc + 31) / 32; }
 __global__ void k_el_geometry(int n, const double* __restrict__ X, double dt, float* __restrict__ G) {
+  dep_wait();
   const size_t nc = (size_t)n * n * n;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 6 * nc) return;
@@ -89,7 +90,7 @@ __global__ void k_el_geometry(int n, const double* __restrict__ X, double dt, fl
 float* element_geometry(const Exec& ex, Arena& ar, int n, const double* X, double dt) {
   const size_t nc = (size_t)n * n * n;
   float* G = ar.alloc<float>(6 * 32 * kElWords * el_blocks(nc));
-  k_el_geometry<<<cdiv((long long)(6 * nc), 256), 256, 0, ex.s>>>(n, X, dt, G);
+  launch_dep(k_el_geometry, cdiv((long long)(6 * nc), 256), 256, 0, ex, n, X, dt, G);
   SK_CHECK_LAUNCH();
   return G;
 }
@@ -251,6 +252,7 @@ constexpr int kElBlock = 192;  // 32 cubes x 6 tetrahedra
 __global__ void __launch_bounds__(kElBlock, 4) k_el_strain(int n, const float* __restrict__ G, float mu,
                                                        const float* __restrict__ x, size_t xs,
                                                        float* __restrict__ part) {
+  dep_wait();
   __shared__ float sh[6][30][32];
   const int nc = n * n * n, m = 2 * n - 1;
   const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(256) k_el_sum(int n, int nb, const float* __re
                                                const float* __restrict__ x, size_t xs, const float* __restrict__ b,
                                                float* __restrict__ y, double* partial, unsigned* counter,
                                                double* dot) {
+  dep_wait();
   const int nc = n * n * n, m = 2 * n - 1;
   const int c = blockIdx.x / nb;
   const int cube = (blockIdx.x - c * nb) * 256 + threadIdx.x;
@@ -380,14 +383,14 @@ void element_strain(const Exec& ex, const ElementOp& e, int k, const float* x, f
   for (int k0 = 0; k0 < k; k0 += e.batch) {
     const int kk = std::min(e.batch, k - k0);
     const size_t o = (size_t)3 * k0 * xs;
-    k_el_strain<<<dim3(cdiv(nc, 32), kk), kElBlock, 0, ex.s>>>(n, e.G, e.mu, x + o, xs, e.part);
+    launch_dep(k_el_strain, dim3(cdiv(nc, 32), kk), kElBlock, 0, ex, n, e.G, e.mu, x + o, xs, e.part);
     SK_CHECK_LAUNCH();
     const dim3 grid(3 * nb, kk);
     if (dot)
-      k_el_sum<true><<<grid, 256, 0, ex.s>>>(n, nb, e.part, x + o, xs, b ? b + o : nullptr, y + o, ds->fused_partial,
+      launch_dep(k_el_sum<true>, grid, 256, 0, ex, n, nb, e.part, x + o, xs, b ? b + o : nullptr, y + o, ds->fused_partial,
                                              ds->fused_counter, dot + k0);
     else
-      k_el_sum<false><<<grid, 256, 0, ex.s>>>(n, nb, e.part, x + o, xs, b ? b + o : nullptr, y + o, nullptr, nullptr,
+      launch_dep(k_el_sum<false>, grid, 256, 0, ex, n, nb, e.part, x + o, xs, b ? b + o : nullptr, y + o, nullptr, nullptr,
                                               nullptr);
     SK_CHECK_LAUNCH();
   }

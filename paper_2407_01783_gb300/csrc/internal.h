@@ -57,6 +57,22 @@ struct FastDiv {
 #endif
 };
 
+// Dependent launches. The solver's work is one chain of kernels, on small meshes
+// and coarse levels of a few microseconds each, so the gap between two of them
+// counts. A kernel launched with launch_dep may be set up on the GPU while its
+// predecessor still runs (CUDA's programmatic stream serialisation, kept as
+// programmatic edges in captured graphs); its first statement dep_wait() waits
+// until the predecessor has finished and its writes are visible, and only then
+// lets its own successor be set up, so at most one grid waits at a time and
+// every kernel still finishes after the one before it. Every thread calls
+// dep_wait() before anything else.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // An NVTX range for the lifetime of the object (solver phases show up as
 // named ranges under a profiler; without one attached the calls do nothing).
 struct NvtxRange {
@@ -96,7 +112,31 @@ struct Exec {
   Prof* prof = nullptr;
   int* flag = nullptr;  // per-context status bits set by kernels (1: Krylov breakdown,
                         // 4: a bounded device wait expired)
+  bool dep = true;      // launch_dep: let a launch be set up while its predecessor runs
 };
+
+#ifdef __CUDACC__
+// Grids of up to a block per SM only: blocks placed early go where there is room
+// at that moment, which unbalances larger grids. Measured limits 0, 152, 456,
+// none (ms): FP64 8^3 86.6, 82.0, 82.1; mixed 12^3 19.3, 17.4, 17.8; FP64 24^3
+// 277.6, 275.1, 283.0, 306; mixed 48^3 103.1, 102.5, 102.8, 103.3; six uneven
+// instances at once 184.5, 182.2, 182.7, 192.5.
+constexpr long long kDepBlocks = 152;
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const Exec& ex, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ex.s;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = ex.dep && (long long)grid.x * grid.y * grid.z <= kDepBlocks ? 1 : 0;
+  SK_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+}
+#endif
 
 // Brackets one launch with events when profiling is on.
 struct ProfScope {

@@ -37,6 +37,7 @@ struct KSeg {
 template <class T>
 __global__ void __launch_bounds__(256) k_kdot(KSeg s, const T* __restrict__ x, const T* __restrict__ y,
                                               double* partial, unsigned* counter, double* out) {
+  dep_wait();
   const int k = blockIdx.y;
   const size_t n = s.len();
   double t = 0.0;
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(256) k_kdot(KSeg s, const T* __restrict__ x, c
 // y_k = a_k x_k + b_k y_k on the chosen segment (x may alias y)
 template <class T>
 __global__ void __launch_bounds__(256) k_kaxpby(KSeg s, KCoefs a, const T* x, KCoefs b, T* y, int* flag) {
+  dep_wait();
   const int k = blockIdx.y;
   __shared__ double ab[2];
   if (threadIdx.x == 0) {
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) k_kaxpby(KSeg s, KCoefs a, const T* x, KC
 // y_k += c_k (a constant per right-hand side, c_k = scale * num_k / den_k)
 template <class T>
 __global__ void __launch_bounds__(256) k_kaddconst(KSeg s, KCoefs c, T* y, int* flag) {
+  dep_wait();
   const int k = blockIdx.y;
   __shared__ double cv;
   if (threadIdx.x == 0) cv = c.value(k, blockIdx.x == 0 ? flag : nullptr);
@@ -92,6 +95,7 @@ __global__ void __launch_bounds__(256) k_kaddconst(KSeg s, KCoefs c, T* y, int* 
 template <class T, int KB>
 __global__ void __launch_bounds__(256) k_kmdot(KSeg s, KBasis<T> V, int J, const T* __restrict__ w, double* partial,
                                                unsigned* counter, double* out, int ld) {
+  dep_wait();
   const int k = blockIdx.y;
   const size_t n = s.len();
   double acc[KB];
@@ -155,6 +159,7 @@ __global__ void __launch_bounds__(256) k_kmdot(KSeg s, KBasis<T> V, int J, const
 template <class T, int KB>
 __global__ void __launch_bounds__(256) k_kmaxpy(KSeg s, KBasis<T> V, int J, const double* h, KHost hc, int ld,
                                                 double sign, T* w) {
+  dep_wait();
   const int k = blockIdx.y;
   __shared__ T c[KB];
   if (threadIdx.x < KB)
@@ -173,6 +178,7 @@ __global__ void __launch_bounds__(256) k_kmaxpy(KSeg s, KBasis<T> V, int J, cons
 }
 
 __global__ void k_ksub(int K, double* out, const double* a, const double* b) {
+  dep_wait();
   const int k = threadIdx.x;
   if (k < K) out[k] = a[k] - b[k];
 }
@@ -202,7 +208,7 @@ void kdot(const Exec& ex, const DotScratch& ds, size_t nu, size_t np, int K, int
   SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kdot: 1 to 8 right-hand sides");
   SK_REQUIRE(ds.k_partial && (long long)gx * K <= ds.k_cap, STOKES_ERR_ARG, "kdot: scratch too small");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * K * len * (y ? 2.0 : 1.0));
-  k_kdot<T><<<dim3(gx, K), 256, 0, ex.s>>>(kseg(nu, np, K, parts), x, y, ds.k_partial, ds.k_counter, out);
+  launch_dep(k_kdot<T>, dim3(gx, K), 256, 0, ex, kseg(nu, np, K, parts), x, y, ds.k_partial, ds.k_counter, out);
   SK_CHECK_LAUNCH();
 }
 
@@ -212,7 +218,7 @@ void kaxpby(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs
   SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kaxpby: 1 to 8 right-hand sides");
   const size_t len = seglen(nu, np, parts);
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * K * len * 3.0);
-  k_kaxpby<T><<<dim3(kgrid(len), K), 256, 0, ex.s>>>(kseg(nu, np, K, parts), a, x, b, y, ex.flag);
+  launch_dep(k_kaxpby<T>, dim3(kgrid(len), K), 256, 0, ex, kseg(nu, np, K, parts), a, x, b, y, ex.flag);
   SK_CHECK_LAUNCH();
 }
 
@@ -221,7 +227,7 @@ void kaddconst(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCo
   SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kaddconst: 1 to 8 right-hand sides");
   const size_t len = seglen(nu, np, parts);
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * K * len * 2.0);
-  k_kaddconst<T><<<dim3(kgrid(len), K), 256, 0, ex.s>>>(kseg(nu, np, K, parts), c, y, ex.flag);
+  launch_dep(k_kaddconst<T>, dim3(kgrid(len), K), 256, 0, ex, kseg(nu, np, K, parts), c, y, ex.flag);
   SK_CHECK_LAUNCH();
 }
 
@@ -239,12 +245,12 @@ void kmdot(const Exec& ex, const DotScratch& ds, size_t nu, size_t np, int K, in
   const KSeg sg = kseg(nu, np, K, 3);
   const dim3 grid(gx, K);
   switch (KB) {
-    case 1: k_kmdot<T, 1><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
-    case 2: k_kmdot<T, 2><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
-    case 4: k_kmdot<T, 4><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
-    case 8: k_kmdot<T, 8><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
-    case 16: k_kmdot<T, 16><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
-    default: k_kmdot<T, 32><<<grid, 256, 0, ex.s>>>(sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    case 1: launch_dep(k_kmdot<T, 1>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    case 2: launch_dep(k_kmdot<T, 2>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    case 4: launch_dep(k_kmdot<T, 4>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    case 8: launch_dep(k_kmdot<T, 8>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    case 16: launch_dep(k_kmdot<T, 16>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
+    default: launch_dep(k_kmdot<T, 32>, grid, 256, 0, ex, sg, B, J, w, ds.k_partial, ds.k_counter, out, ld); break;
   }
   SK_CHECK_LAUNCH();
 }
@@ -265,12 +271,12 @@ void kmaxpy(const Exec& ex, size_t nu, size_t np, int K, int J, const T* const* 
   const KSeg sg = kseg(nu, np, K, 3);
   const dim3 grid(kgrid(len), K);
   switch (pow2_ge(J)) {
-    case 1: k_kmaxpy<T, 1><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
-    case 2: k_kmaxpy<T, 2><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
-    case 4: k_kmaxpy<T, 4><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
-    case 8: k_kmaxpy<T, 8><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
-    case 16: k_kmaxpy<T, 16><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
-    default: k_kmaxpy<T, 32><<<grid, 256, 0, ex.s>>>(sg, B, J, h, hc, ld, sign, w); break;
+    case 1: launch_dep(k_kmaxpy<T, 1>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
+    case 2: launch_dep(k_kmaxpy<T, 2>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
+    case 4: launch_dep(k_kmaxpy<T, 4>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
+    case 8: launch_dep(k_kmaxpy<T, 8>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
+    case 16: launch_dep(k_kmaxpy<T, 16>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
+    default: launch_dep(k_kmaxpy<T, 32>, grid, 256, 0, ex, sg, B, J, h, hc, ld, sign, w); break;
   }
   SK_CHECK_LAUNCH();
 }
@@ -278,7 +284,7 @@ void kmaxpy(const Exec& ex, size_t nu, size_t np, int K, int J, const T* const* 
 void ksub(const Exec& ex, int K, double* out, const double* a, const double* b) {
   SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "ksub: 1 to 8 values");
   ProfScope ps(ex, STOKES_KERNEL_OTHER, 24.0 * K);
-  k_ksub<<<1, 32, 0, ex.s>>>(K, out, a, b);
+  launch_dep(k_ksub, 1, 32, 0, ex, K, out, a, b);
   SK_CHECK_LAUNCH();
 }
 

@@ -371,6 +371,7 @@ template <int G, int NR, class TM, class T, class Epi>
 __global__ void __launch_bounds__(256) k_csr(int rows, const int* __restrict__ rp, const int* __restrict__ col,
                                              const TM* __restrict__ val, const T* __restrict__ x, size_t xs,
                                              Epi epi) {
+  dep_wait();
   constexpr int U = Batch<G>::U;
   int gt = blockIdx.x * blockDim.x + threadIdx.x;
   int row = gt / G, lane = gt & (G - 1);
@@ -435,6 +436,7 @@ template <int G, class T, class Epi>
 __global__ void __launch_bounds__(256) k_bsr3(int rows, const int* __restrict__ rp, const int* __restrict__ col,
                                               const T* __restrict__ v, long long nnz, const T* __restrict__ x,
                                               size_t xs, Epi epi) {
+  dep_wait();
   constexpr int U = Batch<G>::U > 4 ? 4 : Batch<G>::U;
   int gt = blockIdx.x * blockDim.x + threadIdx.x;
   int row = gt / G, lane = gt & (G - 1);
@@ -474,6 +476,7 @@ __global__ void __launch_bounds__(256) k_bsr3_df(int rows, const int* __restrict
                                                  long long nnz, const float* __restrict__ xh,
                                                  const float* __restrict__ xl, size_t xs,
                                                  const double* __restrict__ b, double* __restrict__ y) {
+  dep_wait();
   constexpr int U = 2;
   int gt = blockIdx.x * blockDim.x + threadIdx.x;
   int row = gt / G, lane = gt & (G - 1);
@@ -532,7 +535,7 @@ static void launch_bsr3_df(const Exec& ex, const Csr& m, const float* xh, const 
   const int bs = 256;
   const int grid = cdiv((long long)m.rows * G, bs);
   if (grid == 0) return;
-  k_bsr3_df<G><<<grid, bs, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.v32, m.v32lo, m.nnz, xh, xl, m.cols, b, y);
+  launch_dep(k_bsr3_df<G>, grid, bs, 0, ex, m.rows, m.rowptr, m.col, m.v32, m.v32lo, m.nnz, xh, xl, m.cols, b, y);
   SK_CHECK_LAUNCH();
 }
 
@@ -565,6 +568,7 @@ __global__ void __launch_bounds__(256) k_bsr3_dot(int rows, const int* __restric
                                                   const T* __restrict__ v, long long nnz, const T* __restrict__ x,
                                                   size_t xs, T* __restrict__ y, double* partial, unsigned* counter,
                                                   double* dot) {
+  dep_wait();
   constexpr int U = Batch<G>::U > 4 ? 4 : Batch<G>::U;
   // a grid of one resident wave walks the row groups (grid stride), so the
   // grid sum below takes one counter increment per resident block, not per
@@ -631,7 +635,7 @@ static void launch_bsr3_dot(const Exec& ex, const Csr& m, const T* x, T* y, cons
   if (!slot) slot = resident_grid(k_bsr3_dot<G, T>, 256, 1 << 30);
   const int grid = std::min(want, slot);
   SK_REQUIRE(ds.fused_partial && grid <= ds.fused_cap, STOKES_ERR_ARG, "fused dot scratch too small");
-  k_bsr3_dot<G, T><<<grid, 256, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, (size_t)m.cols, y,
+  launch_dep(k_bsr3_dot<G, T>, grid, 256, 0, ex, m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, (size_t)m.cols, y,
                                            ds.fused_partial, ds.fused_counter, dot);
   SK_CHECK_LAUNCH();
 }
@@ -651,6 +655,7 @@ template <int G, int K, class T, class Epi>
 __global__ void __launch_bounds__(256) k_b(int rows, const int* __restrict__ rp, const int* __restrict__ col,
                                            const T* __restrict__ v, long long nnz, const T* __restrict__ x, size_t xs,
                                            Epi epi) {
+  dep_wait();
   constexpr int U = Batch<G>::U;
   int gt = blockIdx.x * blockDim.x + threadIdx.x;
   int row = gt / G, lane = gt & (G - 1);
@@ -693,6 +698,7 @@ template <int G, int K, class T, class Epi>
 __global__ void __launch_bounds__(256) k_bt(int rows, const int* __restrict__ rp, const int* __restrict__ col,
                                             const T* __restrict__ v, long long nnz, const T* __restrict__ x, size_t xs,
                                             Epi epi) {
+  dep_wait();
   constexpr int U = Batch<G>::U;
   int gt = blockIdx.x * blockDim.x + threadIdx.x;
   int row = gt / G, lane = gt & (G - 1);
@@ -761,6 +767,7 @@ constexpr int kStUnroll = SK_ST_UNROLL;
 template <int NR, class TM, class T, class Epi>
 __global__ void __launch_bounds__(SK_ST_BLOCK) k_stencil(const StArgs a, const TM* __restrict__ v, const T* __restrict__ x,
                                                  size_t xs, Epi epi) {
+  dep_wait();
   int c, r;
   if (!st_locate(a, c, r)) return;
   int i, qx, qy, qz;
@@ -829,7 +836,7 @@ static void launch_stencil(const Exec& ex, const StencilOp& so, int nr, const T*
   size_t xs = 0;
   for (int c = 0; c < so.ncls; ++c) xs += so.rows[c];
   (void)nr;
-  k_stencil<Epi::nr, T, T, Epi><<<grid, bs, 0, ex.s>>>(a, so.template v<T>(), x, xs, epi);
+  launch_dep(k_stencil<Epi::nr, T, T, Epi>, grid, bs, 0, ex, a, so.template v<T>(), x, xs, epi);
   SK_CHECK_LAUNCH();
 }
 
@@ -857,20 +864,20 @@ static void launch_g(const Exec& ex, const Csr& m, Shape sh, const T* x, const E
   if (grid == 0) return;
   switch (sh) {
     case SH_CSR:
-      k_csr<G, Epi::nr, T, T, Epi><<<grid, bs, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.template v<T>(), x, m.cols, epi);
+      launch_dep(k_csr<G, Epi::nr, T, T, Epi>, grid, bs, 0, ex, m.rows, m.rowptr, m.col, m.template v<T>(), x, m.cols, epi);
       break;
     case SH_BSR3:
       if constexpr (Epi::nr == 3)
-        k_bsr3<G, T, Epi><<<grid, bs, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, m.cols, epi);
+        launch_dep(k_bsr3<G, T, Epi>, grid, bs, 0, ex, m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, m.cols, epi);
       break;
     case SH_B:
       if constexpr (Epi::nr == 1 || Epi::nr == 4)
-        k_b<G, Epi::nr, T, Epi><<<grid, bs, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, m.cols,
+        launch_dep(k_b<G, Epi::nr, T, Epi>, grid, bs, 0, ex, m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x, m.cols,
                                                        epi);
       break;
     case SH_BT:
       if constexpr (Epi::nr == 3 || Epi::nr == 12)
-        k_bt<G, Epi::nr / 3, T, Epi><<<grid, bs, 0, ex.s>>>(m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x,
+        launch_dep(k_bt<G, Epi::nr / 3, T, Epi>, grid, bs, 0, ex, m.rows, m.rowptr, m.col, m.template v<T>(), m.nnz, x,
                                                             m.cols, epi);
       break;
   }
@@ -1151,6 +1158,7 @@ template <class T> void bt_apply(const Exec& ex, const Csr& m, const T* x, T* y,
 // coarse dense inverse applied to NR right-hand sides: one warp per row
 template <int NR, class T, bool IL = false>
 __global__ void k_dense(const T* __restrict__ M, int m, const T* __restrict__ b, T* __restrict__ y) {
+  dep_wait();
   // component-major right-hand sides: component r of row j at r * m + j
   // (IL: node-interleaved, at j * NR + r)
   int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1178,8 +1186,8 @@ template <class T> void dense_apply(const Exec& ex, const T* Minv, int m, int nr
   int grid = cdiv(m, 8);
   with_nr(nr, [&](auto NRc) {
     constexpr int NR = decltype(NRc)::value;
-    if (il) k_dense<NR, T, true><<<grid, 256, 0, ex.s>>>(Minv, m, b, y);
-    else k_dense<NR, T, false><<<grid, 256, 0, ex.s>>>(Minv, m, b, y);
+    if (il) launch_dep(k_dense<NR, T, true>, grid, 256, 0, ex, Minv, m, b, y);
+    else launch_dep(k_dense<NR, T, false>, grid, 256, 0, ex, Minv, m, b, y);
   });
   SK_CHECK_LAUNCH();
 }
@@ -1268,6 +1276,7 @@ void autotune_group(const Exec& ex, Csr& m, int nr, int kind, int k) {
   SK_CUDA(cudaEventCreate(&e0));
   SK_CUDA(cudaEventCreate(&e1));
   Exec plain{ex.s, nullptr};
+  plain.dep = false;  // time launches on their own, not overlapped with the next
   float best = FLT_MAX;
   int bestg = slot ? slot : m.group;
   const int gs[5] = {2, 4, 8, 16, 32};

@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(kSymBlock) k_sym3(const Sym3Args a, int nvb, c
                                                    const T* __restrict__ x, size_t xs, const T* __restrict__ b,
                                                    T* __restrict__ y, double* partial, unsigned* counter,
                                                    double* dot) {
+  dep_wait();
   static_assert(!DOT || K == 1, "fused dot: one right-hand side");
   const int lane = (int)threadIdx.x % G;
   double part = 0.0;
@@ -236,6 +237,7 @@ __global__ void __launch_bounds__(kSymBlock) k_sym3_df(const Sym3Args a, const f
                                                       const float* __restrict__ vl, const float* __restrict__ xh,
                                                       const float* __restrict__ xl, size_t xs,
                                                       const double* __restrict__ b, double* __restrict__ y) {
+  dep_wait();
   const SymRow R = sym3_locate<G>(a, (int)blockIdx.x);
   const int lane = (int)threadIdx.x % G;
   const int c = R.c;
@@ -360,10 +362,10 @@ static void sym3_launch_g(const Exec& ex, const Csr& m, const double* x, double*
   const int grid = std::min(nvb, w);
   if (dot) {
     SK_REQUIRE(ds && ds->fused_partial && grid <= ds->fused_cap, STOKES_ERR_ARG, "fused dot scratch too small");
-    k_sym3<G, U, double, true><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y,
+    launch_dep(k_sym3<G, U, double, true>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y,
                                                     ds->fused_partial, ds->fused_counter, dot);
   } else {
-    k_sym3<G, U, double, false><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
+    launch_dep(k_sym3<G, U, double, false>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
                                                      nullptr, nullptr);
   }
   SK_CHECK_LAUNCH();
@@ -385,7 +387,7 @@ void sym3_launch4(const Exec& ex, const Csr& m, const double* x, double* y, cons
     w = std::max(1, sms * std::max(1, occ));
   }
   const int grid = std::min(nvb, w);
-  k_sym3<1, 2, double, false, 4><<<grid, kSymBlock, 0, ex.s>>>(a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
+  launch_dep(k_sym3<1, 2, double, false, 4>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
                                                        nullptr, nullptr);
   SK_CHECK_LAUNCH();
 }
@@ -409,7 +411,7 @@ static void sym3_df_g(const Exec& ex, const Csr& m, const float* xh, const float
   const Sym3Args a = sym3_args(so, G);
   const int grid = sym3_blocks(so, a);
   if (grid == 0) return;
-  k_sym3_df<G><<<grid, kSymBlock, 0, ex.s>>>(a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
+  launch_dep(k_sym3_df<G>, grid, kSymBlock, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
   SK_CHECK_LAUNCH();
 }
 
@@ -419,7 +421,7 @@ void sym3_residual_df4(const Exec& ex, const Csr& m, const float* xh, const floa
   const Sym3Args a = sym3_args(so, 1);
   const int grid = sym3_blocks(so, a);
   if (grid == 0) return;
-  k_sym3_df<1, 4><<<grid, kSymBlock, 0, ex.s>>>(a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
+  launch_dep(k_sym3_df<1, 4>, grid, kSymBlock, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
   SK_CHECK_LAUNCH();
 }
 

@@ -26,6 +26,7 @@ struct ProlongArgs {
 template <int NR, bool IL>
 __global__ void __launch_bounds__(256) k_prolong_p2(const ProlongArgs a, const float* __restrict__ x, size_t xs,
                                                    float* __restrict__ y, size_t ys) {
+  dep_wait();
   const int t = blockIdx.x * 256 + threadIdx.x;
   if (t >= a.total) return;
   const int z = a.by_mm.div(t), tz = t - z * a.by_mm.d, yy = a.by_m.div(tz);
@@ -115,8 +116,8 @@ void prolong_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* y
                 FastDiv(D), sm ? *sm : SplitMap{}, sm ? 1 : 0};
   const int grid = cdiv(a.total, 256);
   const size_t xs = (size_t)mc * mc * mc, ys = (size_t)a.total;
-  if (nr == 3 && !il) k_prolong_p2<3, false><<<grid, 256, 0, ex.s>>>(a, x, xs, y, ys);
-  else if (nr == 12 && il) k_prolong_p2<12, true><<<grid, 256, 0, ex.s>>>(a, x, xs, y, ys);
+  if (nr == 3 && !il) launch_dep(k_prolong_p2<3, false>, grid, 256, 0, ex, a, x, xs, y, ys);
+  else if (nr == 12 && il) launch_dep(k_prolong_p2<12, true>, grid, 256, 0, ex, a, x, xs, y, ys);
   else throw Error(STOKES_ERR_ARG, "P2 transfer: 3 component-major or 12 interleaved components");
   SK_CHECK_LAUNCH();
 }
@@ -196,6 +197,7 @@ static RestrictArgs restrict_args(int nc) {
 template <int NR, bool IL>
 __global__ void __launch_bounds__(256) k_restrict_p2(const RestrictArgs a, const float* __restrict__ x, size_t xs,
                                                     float* __restrict__ y, size_t ys) {
+  dep_wait();
   constexpr int L = IL ? NR / 4 : 1;  // lanes per node
   using V = typename std::conditional<IL, float4, float>::type;
   __shared__ V sh[8][32];
@@ -260,9 +262,9 @@ bool restrict_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* 
   if (sm) a.sm = *sm;
   const size_t xs = (size_t)a.mf * a.mf * a.mf, ys = (size_t)a.mc * a.mc * a.mc;
   const int rows = nc * nc * nc;  // most of any class
-  if (nr == 3 && !il) k_restrict_p2<3, false><<<dim3(cdiv(rows, 32), 8, 3), 256, 0, ex.s>>>(a, x, xs, y, ys);
+  if (nr == 3 && !il) launch_dep(k_restrict_p2<3, false>, dim3(cdiv(rows, 32), 8, 3), 256, 0, ex, a, x, xs, y, ys);
   else if (nr == 12 && il)
-    k_restrict_p2<12, true><<<dim3(cdiv(3LL * rows, 32), 8), 256, 0, ex.s>>>(a, x, xs, y, ys);
+    launch_dep(k_restrict_p2<12, true>, dim3(cdiv(3LL * rows, 32), 8), 256, 0, ex, a, x, xs, y, ys);
   else throw Error(STOKES_ERR_ARG, "P2 transfer: 3 component-major or 12 interleaved components");
   SK_CHECK_LAUNCH();
   return true;
