@@ -106,7 +106,7 @@ typedef struct {
                             its inner velocity solves get max(inner_tol,
                             pass_tol/30). Default 3e-2. */
   int format;            /* 0: stencil-structured storage for A~_3, eps M_Q + L_Q,
-                            M_Q, L_Q on levels with >= 2^18 rows, CSR below; the
+                            M_Q, L_Q on every level (see stencil_min_rows); the
                             strain-form A in symmetric stencil storage (diagonal
                             and upper 3x3 blocks only: half the matrix bytes)
                             for its FP64 products and the double-float
@@ -154,11 +154,12 @@ typedef struct {
                             An interval far below the spectrum makes the
                             V-cycle indefinite; the Krylov solvers then report
                             STOKES_ERR_BREAKDOWN. */
-  int sym_batch;         /* symmetric (FP64) A products: block entries whose loads one
-                            thread issues before using them (2, 4 or 8; 0:
-                            default 8) */
-  int stencil_min_rows;  /* formats 0 and 3: levels with at least this many rows
-                            use stencil storage (0: 2^18) */
+  int sym_batch;         /* symmetric (FP64) A products: block entries whose loads
+                            one thread issues before using them (2, 4 or 8; 0:
+                            default 2; 8 is taken as 4) */
+  int stencil_min_rows;  /* formats 0 and 3: with one right-hand side, levels with
+                            at least this many rows use stencil storage (0:
+                            every level) */
   int host_wait;         /* how the host thread waits for the device scalars
                             it reads: 0 spins (lowest latency; the default),
                             1 sleeps until the GPU signals (blocking-sync

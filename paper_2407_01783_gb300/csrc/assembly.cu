@@ -1031,6 +1031,8 @@ StArgs stencil_args(const StencilOp& so, int block, int rows_per_thread, bool sp
     a.pext[c] = so.pext[c];
     a.prows[c] = so.prows[c];
     for (int k = 0; k < 3; ++k) a.ext[c][k] = so.ext[c][k], a.q0[c][k] = so.q0[c][k];
+    a.Mx[c] = FastDiv(std::max(1, so.ext[c][0])).M;
+    a.My[c] = FastDiv(std::max(1, so.ext[c][1])).M;
     a.bbeg[c] = b;
     b += cdiv(so.prows[c] / rows_per_thread, block);
   }

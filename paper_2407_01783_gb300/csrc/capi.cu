@@ -240,12 +240,13 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
   }
   if (c.opt.format != 1) {
     auto add = [&](Csr& m, int p2, int nn) {
-      const int min_rows = c.opt.stencil_min_rows > 0 ? c.opt.stencil_min_rows : kStencilMinRows;
+      // every level (the kernels split short levels' rows over warps), unless
+      // the caller set a size from which on one right-hand side uses it
       const bool by_size = c.opt.format == 0 || c.opt.format == 3;
-      if (by_size && m.rows < std::min(min_rows, kStencilMinRowsIL)) return;
+      const int min_rows = by_size ? c.opt.stencil_min_rows : 0;
       c.stencils.emplace_back(stencil_from_csr(c.ex, c.arena, st, p2, nn, m));
       m.st = c.stencils.back().get();
-      m.st_min_single = by_size ? min_rows : 0;
+      m.st_min_single = min_rows;
     };
     for (Level& L : c.lv) {
       add(L.A3, 1, L.n);
@@ -385,12 +386,7 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
     m.group4 = probe.group4;
   };
   tune(c.A, 3, 1);
-  // threads per row of the symmetric A products: one (measured fastest inside
-  // the solve at 48^3: 201 us against 232, 318, 508 us for 2, 4, 8) unless set
-  if (c.A.sym) {
-    c.symA->group = c.opt.spmv_group > 0 ? std::min(8, c.A.group) : 1;
-    c.symA->batch = c.opt.sym_batch > 0 ? c.opt.sym_batch : 8;
-  }
+  if (c.A.sym) c.symA->batch = c.opt.sym_batch > 0 ? c.opt.sym_batch : 2;
   if (!c.divB) {
     tune(c.B, 1, 2);
     tune(c.Bt, 3, 3);

@@ -194,6 +194,7 @@ struct StArgs {
   int rows[8], ext[8][3], q0[8][3], S[8], Sreal[8], dbeg[8], pext[8], prows[8];
   long long voff[8];
   int bbeg[9];
+  unsigned long long Mx[8], My[8];  // FastDiv multipliers of ext[c][0], ext[c][1]
   signed char d[kMaxStencil][3];
   int lin[kMaxStencil];
 };
@@ -316,8 +317,7 @@ struct Sym3Op {
   long long lbase[kMaxSym] = {};      // voff[class j] + 9 * (entry -o of class j) * prows[class j]
   signed char ldel[kMaxSym][3] = {};  // position of j in its class minus position of i in its class
   long long total = 0;                // stored values (9 per stored block)
-  int group = 1;                      // threads per row of the products (1, 2, 4 or 8)
-  int batch = 8;                      // entries whose loads a lane issues together (2, 4 or 8)
+  int batch = 2;                      // entries whose loads a lane issues together (2; 4 from sym_batch 4 on)
   double* v64 = nullptr;
   float* v32 = nullptr;
   float* v32lo = nullptr;             // FP32(v64 - v32): double-float residual
@@ -367,7 +367,8 @@ struct Csr {
   int group4 = 0; // threads per row of four-right-hand-side products (B, B^T; 0: group)
   const StencilOp* st = nullptr;  // same matrix in stencil storage (used when set, see st_min_single)
   int st_min_single = 0;          // component-major products (one right-hand side) use the stencil
-                                  // storage only on matrices with at least this many rows
+                                  // storage only on matrices with at least this many rows (option
+                                  // stencil_min_rows)
   const Sym3Op* sym = nullptr;    // 3x3-block matrix in symmetric stencil storage: used for the
                                   // double-float residual, and for all products if sym_products
   bool sym_products = false;
@@ -735,13 +736,18 @@ int bsr3_dot_grid(const Csr& m);
 // dots() (velocity-sized vectors of the inner solves); shorter ones
 // (pressure-sized, the outer Schur iteration) accumulate in FP64 throughout.
 constexpr size_t kCompensatedMin = (size_t)1 << 20;
-// Stencil storage is used on levels with at least this many rows; smaller
-// grids are latency-bound with one thread per row and stay CSR.
-constexpr int kStencilMinRows = 1 << 18;
-// With several right-hand sides (node-interleaved vectors, 4 or 12 values per
-// row) a row carries enough work that the stencil kernel already pays from
-// this size on.
-constexpr int kStencilMinRowsIL = 1 << 15;
+// Rows below which the stencil kernels spread a row's entries over 8, 4 and 2
+// warps (k_stencil_w): FP32 component-major, FP64, interleaved. Whole solves in
+// ms with the lines (powers of two) set to ...: FP32, 48^3: {14, 16, 18} 102.5,
+// {15, 16, 19} 101.2, {13, 15, 17} 102.7, {15, 18, 20} 114; FP64, 24^3:
+// {14, 16, 17} 277, {15, 17, 18} 274, {13, 17, 18} 274; interleaved, six systems
+// at 25^3 / four at 40^3 / the uneven batch: {16, 18, 18} 166 / 90 / 185,
+// {14, 16, 18} 168 / 92 / 182, {16, 18, 20} 168 / 86 / 189, {13, 15, 15} 178 / 93
+// / 181, a thread per row 237 / 102 / 184. Against CSR on the levels below 2^18
+// rows: FP64 24^3 353 -> 275, mixed 33^3 66 -> 62.5.
+constexpr long long kStencilSplit32[3] = {1 << 15, 1 << 16, 1 << 19};
+constexpr long long kStencilSplit64[3] = {1 << 15, 1 << 17, 1 << 18};
+constexpr long long kStencilSplitIL[3] = {1 << 16, 1 << 18, 1 << 18};
 // out[i] = sum_j x_i[j] * y_i[j] for i < k (y_i == nullptr means all ones).
 // Accumulation of FP32 dot products: kDotAuto = compensated FP32 partial sums
 // for vectors of at least kCompensatedMin entries, kDotFast = compensated for
@@ -860,6 +866,11 @@ template <class T> void kdot(const Exec& ex, const DotScratch& ds, size_t nu, si
 // y_k = a_k x_k + b_k y_k over the segment
 template <class T> void kaxpby(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs& a, const T* x,
                                const KCoefs& b, T* y);
+// one CG update of K plain blocks of length n: x_k += a_k d_k, r_k -= a_k q_k
+// and, with rr, rr[k] = r_k . r_k
+template <class T>
+void kcg_update(const Exec& ex, const DotScratch& ds, size_t n, int K, const KCoefs& a, const T* d, T* x, const T* q,
+                T* r, double* rr);
 // y_k += c_k over the segment
 template <class T> void kaddconst(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs& c, T* y);
 // Arnoldi helpers over whole segments (parts = 3) of J <= kMaxBasisK

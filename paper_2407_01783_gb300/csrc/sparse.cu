@@ -89,9 +89,10 @@ template <class T, int NR> struct EpiStore {
   static constexpr bool il = false;
   T* y;
   size_t ns;
+  __device__ __forceinline__ void comp(int row, int r, T v) const { y[r * ns + row] = v; }
   __device__ __forceinline__ void operator()(int row, const T* acc) const {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) y[r * ns + row] = acc[r];
+    for (int r = 0; r < NR; ++r) comp(row, r, acc[r]);
   }
 };
 template <class T, int NR> struct EpiAdd {
@@ -99,9 +100,10 @@ template <class T, int NR> struct EpiAdd {
   static constexpr bool il = false;
   T* y;
   size_t ns;
+  __device__ __forceinline__ void comp(int row, int r, T v) const { y[r * ns + row] += v; }
   __device__ __forceinline__ void operator()(int row, const T* acc) const {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) y[r * ns + row] += acc[r];
+    for (int r = 0; r < NR; ++r) comp(row, r, acc[r]);
   }
 };
 template <class T, int NR> struct EpiResid {
@@ -110,9 +112,10 @@ template <class T, int NR> struct EpiResid {
   const T* b;
   T* y;
   size_t ns;
+  __device__ __forceinline__ void comp(int row, int r, T v) const { y[r * ns + row] = b[r * ns + row] - v; }
   __device__ __forceinline__ void operator()(int row, const T* acc) const {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) y[r * ns + row] = b[r * ns + row] - acc[r];
+    for (int r = 0; r < NR; ++r) comp(row, r, acc[r]);
   }
 };
 template <class T, int NR> struct EpiAxpy {
@@ -145,16 +148,16 @@ template <class T, int NR> struct EpiCheb {
   const T* dinv;
   T c1, c2;
   size_t ns;
+  __device__ __forceinline__ void comp(int row, int r, T v) const {
+    const size_t i = r * ns + row;
+    const T res = b[i] - v;
+    const T dn = c1 * d[i] + c2 * dinv[row] * res;
+    d[i] = dn;
+    xout[i] = xin[i] + dn;
+  }
   __device__ __forceinline__ void operator()(int row, const T* acc) const {
-    T di = dinv[row];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      size_t i = r * ns + row;
-      T res = b[i] - acc[r];
-      T dn = c1 * d[i] + c2 * di * res;
-      d[i] = dn;
-      xout[i] = xin[i] + dn;
-    }
+    for (int r = 0; r < NR; ++r) comp(row, r, acc[r]);
   }
 };
 
@@ -315,17 +318,18 @@ template <class T, int NR> struct EpiChebFirst {
   T s0, c1, c2;
   size_t ns;
   __device__ __forceinline__ T gather_scale(size_t col) const { return s0 * dinv[col]; }
-  __device__ __forceinline__ void operator()(int row, const T* acc) const {
+  __device__ __forceinline__ void comp(int row, int r, T v) const {
     const T di = dinv[row];
+    const size_t i = r * ns + row;
+    const T bv = b[i];
+    const T x1 = s0 * di * bv;
+    const T dn = c1 * x1 + c2 * di * (bv - v);
+    d[i] = dn;
+    xout[i] = x1 + dn;
+  }
+  __device__ __forceinline__ void operator()(int row, const T* acc) const {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const size_t i = r * ns + row;
-      const T bv = b[i];
-      const T x1 = s0 * di * bv;
-      const T dn = c1 * x1 + c2 * di * (bv - acc[r]);
-      d[i] = dn;
-      xout[i] = x1 + dn;
-    }
+    for (int r = 0; r < NR; ++r) comp(row, r, acc[r]);
   }
 };
 template <class E, class = void> struct is_first : std::false_type {};
@@ -826,16 +830,115 @@ __global__ void __launch_bounds__(SK_ST_BLOCK) k_stencil(const StArgs a, const T
   epi(row, acc);
 }
 
+// The same with the entry groups of a row spread over the W warps of a block of
+// 32 rows (warp w takes groups w, w + W, ...) and the W partial sums added in
+// shared memory: a thread per row leaves small levels latency-bound (one long
+// chain of loads per row, or in FP64 of multiply-adds) and large ones idle in
+// their last wave. Component-major rows end with a warp per component.
+template <int NR, int W, class TM, class T, class Epi>
+__global__ void __launch_bounds__(32 * W) k_stencil_w(const StArgs a, const TM* __restrict__ v,
+                                                      const T* __restrict__ x, size_t xs, Epi epi) {
+  dep_wait();
+  __shared__ T sh[W][NR][32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int c = 0;
+#pragma unroll 1
+  while (c + 1 < a.ncls && (int)blockIdx.x >= a.bbeg[c + 1]) ++c;
+  const int r = ((int)blockIdx.x - a.bbeg[c]) * 32 + lane;
+  const bool live = r < a.rows[c];
+  const int rr = live ? r : a.rows[c] - 1;
+  const int line = (int)((rr * a.Mx[c]) >> 44), iz = (int)((line * a.My[c]) >> 44);  // FastDiv by the class's extents
+  const int row = st_index(a, a.q0[c][0] + 2 * (rr - line * a.ext[c][0]), a.q0[c][1] + 2 * (line - iz * a.ext[c][1]),
+                           a.q0[c][2] + 2 * iz);
+  T acc[NR];
+#pragma unroll
+  for (int q = 0; q < NR; ++q) acc[q] = T(0);
+  using V4 = typename Vec4<TM>::type;
+  const V4* vr = reinterpret_cast<const V4*>(v + a.voff[c]) + rr;
+  const size_t rc = (size_t)a.prows[c];
+  const int S4 = a.S[c] / kStencilVec, db = a.dbeg[c], last = (int)xs - 1;
+#pragma unroll 2
+  for (int e4 = w; e4 < S4; e4 += W) {
+    const V4 w4 = vr[e4 * rc];
+    const TM wv[4] = {w4.x, w4.y, w4.z, w4.w};
+    size_t cc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cc[j] = (size_t)min(max(row + a.lin[db + 4 * e4 + j], 0), last);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      T xv[NR];
+      if constexpr (Epi::il) {
+        ldv<T, NR>(x + cc[j] * NR, xv);
+      } else {
+#pragma unroll
+        for (int q = 0; q < NR; ++q) xv[q] = x[q * xs + cc[j]];
+      }
+      if constexpr (is_first<Epi>::value) {
+        const T f = epi.gather_scale(cc[j]);
+#pragma unroll
+        for (int q = 0; q < NR; ++q) xv[q] *= f;
+      }
+#pragma unroll
+      for (int q = 0; q < NR; ++q) acc[q] += (T)wv[j] * xv[q];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NR; ++q) sh[w][q][lane] = acc[q];
+  __syncthreads();
+  auto sum = [&](int q) {
+    T s[W];
+#pragma unroll
+    for (int u = 0; u < W; ++u) s[u] = sh[u][q][lane];
+#pragma unroll
+    for (int o = W / 2; o; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < o; ++u) s[u] += s[u + o];
+    return s[0];
+  };
+  if constexpr (Epi::il) {
+    if (w == 0 && live) {
+#pragma unroll
+      for (int q = 0; q < NR; ++q) acc[q] = sum(q);
+      epi(row, acc);
+    }
+  } else {
+    for (int q = w; q < NR; q += W) {
+      const T s = sum(q);
+      if (live) epi.comp(row, q, s);
+    }
+  }
+}
+
+// Warps per 32 rows (the lines and their measurements: internal.h)
+template <class T> static inline int stencil_warps(long long rows, bool il) {
+  const long long* lines = il ? kStencilSplitIL : (sizeof(T) == 8 ? kStencilSplit64 : kStencilSplit32);
+  for (int k = 0; k < 3; ++k)
+    if (rows < lines[k]) return 8 >> k;
+  return 1;
+}
+
+template <int W, class T, class Epi>
+static void launch_stencil_w(const Exec& ex, const StencilOp& so, const T* x, const Epi& epi, bool split, size_t xs) {
+  const StArgs a = stencil_args(so, 32, 1, split);
+  const int grid = a.bbeg[so.ncls];
+  if (grid == 0) return;
+  launch_dep(k_stencil_w<Epi::nr, W, T, T, Epi>, grid, 32 * W, 0, ex, a, so.template v<T>(), x, xs, epi);
+}
+
 template <class T, class Epi>
 static void launch_stencil(const Exec& ex, const StencilOp& so, int nr, const T* x, const Epi& epi,
                            bool split = false) {
+  size_t xs = 0;
+  for (int c = 0; c < so.ncls; ++c) xs += so.rows[c];
+  (void)nr;
+  const int W = stencil_warps<T>((long long)xs, Epi::il);
+  if (W == 8) return launch_stencil_w<8>(ex, so, x, epi, split, xs);
+  if (W == 4) return launch_stencil_w<4>(ex, so, x, epi, split, xs);
+  if (W == 2) return launch_stencil_w<2>(ex, so, x, epi, split, xs);
   const int bs = SK_ST_BLOCK;
   StArgs a = stencil_args(so, bs, kStencilRows, split);
   int grid = a.bbeg[so.ncls];
   if (grid == 0) return;
-  size_t xs = 0;
-  for (int c = 0; c < so.ncls; ++c) xs += so.rows[c];
-  (void)nr;
   launch_dep(k_stencil<Epi::nr, T, T, Epi>, grid, bs, 0, ex, a, so.template v<T>(), x, xs, epi);
   SK_CHECK_LAUNCH();
 }

@@ -32,21 +32,19 @@ struct Sym3Args {
   signed char ldel[kMaxSym][3];
 };
 
-constexpr int kSymBlock = 128;
+constexpr int kSymRows = 32;  // rows per block
 
-// G threads share a row (G in {1, 2, 4, 8}), so a block covers 128 / G rows
-static Sym3Args sym3_args(const Sym3Op& so, int G) {
+static Sym3Args sym3_args(const Sym3Op& so) {
   Sym3Args a;
   std::memset(&a, 0, sizeof(a));
   a.m = 2 * so.n - 1;
   a.hiq = 2 * so.n - 1;
-  const int rows_per_block = kSymBlock / G;
   for (int c = 0; c < 8; ++c) {
     for (int k = 0; k < 3; ++k) a.ext[c][k] = so.ext[c][k], a.q0[c][k] = so.q0[c][k];
     a.pext[c] = so.pext[c];
     a.prows[c] = so.prows[c];
     a.voff[c] = so.voff[c];
-    a.nb[c] = cdiv((long long)so.pext[c] * so.ext[c][1], rows_per_block);
+    a.nb[c] = cdiv((long long)so.pext[c] * so.ext[c][1], kSymRows);
   }
   for (int c = 0; c < 9; ++c) a.ubeg[c] = so.ubeg[c], a.lbeg[c] = so.lbeg[c];
   // classes with an odd z coordinate (bit 2 set) have rows on odd planes
@@ -68,16 +66,15 @@ static Sym3Args sym3_args(const Sym3Op& so, int G) {
 // n odd planes (qz = 1, 3, ..., 2n-1) and n-1 even planes (qz = 2, ..., 2n-2),
 // interleaved: odd plane k, even plane k, odd plane k+1, ...
 static int sym3_blocks(const Sym3Op& so, const Sym3Args& a) { return so.n * a.bo + (so.n - 1) * a.be; }
-// most blocks any thread-per-row width launches (8 threads per row)
-int sym3_grid(const Sym3Op& so) { return sym3_blocks(so, sym3_args(so, 8)); }
+int sym3_grid(const Sym3Op& so) { return sym3_blocks(so, sym3_args(so)); }
 
 struct SymRow {
   int c, ix, iy, iz, pr, row, qx, qy, qz;
   bool valid;
 };
 
-template <int G>
-__device__ __forceinline__ SymRow sym3_locate(const Sym3Args& a, int vb) {
+// row `slot` of virtual block vb, `rows` rows per block
+__device__ __forceinline__ SymRow sym3_locate(const Sym3Args& a, int vb, int rows, int slot) {
   SymRow r;
   const int pair = vb / (a.bo + a.be);
   int rem = vb - pair * (a.bo + a.be);
@@ -89,7 +86,7 @@ __device__ __forceinline__ SymRow sym3_locate(const Sym3Args& a, int vb) {
   r.c = c;
   r.iz = pair;  // odd planes: qz = 1 + 2 pair; even planes: qz = 2 + 2 pair
   const int plane = a.pext[c] * a.ext[c][1];
-  const int t = rem * (kSymBlock / G) + (int)threadIdx.x / G;
+  const int t = rem * rows + slot;
   r.valid = t < plane;
   const int tt = r.valid ? t : 0;
   r.ix = tt % a.pext[c];
@@ -106,18 +103,14 @@ __device__ __forceinline__ bool sym3_inside(const Sym3Args& a, int x, int y, int
   return x >= 1 && x <= a.hiq && y >= 1 && y <= a.hiq && z >= 1 && z <= a.hiq;
 }
 
-// Batched loads (as in the CSR kernels): a lane first issues the value loads
-// of U entries (entries lane, lane + G, ..., lane + (U-1) G of its row), then
-// their x gathers, then the FMAs, so that U block loads per lane are in flight
-// per HBM round trip. Entries past the end re-read a valid entry and weigh 0.
-template <int G>
-struct SymBatch {
-  static constexpr int U = 8 / G;
-};
-
-// this lane's share of acc[3k + r] = sum over the row's blocks of
+// Batched loads (as in the CSR kernels): a thread first issues the value loads of
+// U entries (entries lane, lane + G, ..., lane + (U-1) G of its row, lane the
+// thread's warp in the block), then their x gathers, then the FMAs, so that U
+// block loads per thread are in flight per HBM round trip. Entries past the end
+// re-read a valid entry and weigh 0.
+// this thread's share of acc[3k + r] = sum over the row's blocks of
 // A(i, j)_{r q} x_k,j[q] for K right-hand sides (x: 3K component-major
-// components), U entries' loads in flight per lane; each block is read once
+// components), U entries' loads in flight; each block is read once
 // for all K
 template <int G, int U, int K, class T>
 __device__ __forceinline__ void sym3_row(const Sym3Args& a, const SymRow& R, int lane, const T* __restrict__ v,
@@ -192,39 +185,47 @@ __device__ __forceinline__ void sym3_row(const Sym3Args& a, const SymRow& R, int
   }
 }
 
-// y = A x (b == nullptr) or y = b - A x; with DOT, *dot = x . (A x) over all rows
+// y = A x (b == nullptr) or y = b - A x; with DOT, *dot = x . (A x) over all rows.
+// A block takes 32 rows; its warp w the entries w, w + W, ... of each, the
+// partial sums are added in shared memory and a warp per component finishes.
 // Blocks walk the virtual blocks (plane order) with a grid stride; the dot
 // variant runs one resident wave so that its grid sum takes one counter
 // increment per resident block.
 // K right-hand sides: x, b, y hold 3K component-major components (the dot
 // variant is K = 1 only)
-template <int G, int U, class T, bool DOT, int K = 1>
-__global__ void __launch_bounds__(kSymBlock) k_sym3(const Sym3Args a, int nvb, const T* __restrict__ v,
-                                                   const T* __restrict__ x, size_t xs, const T* __restrict__ b,
-                                                   T* __restrict__ y, double* partial, unsigned* counter,
-                                                   double* dot) {
+template <int W, int U, class T, bool DOT, int K = 1>
+__global__ void __launch_bounds__(32 * W) k_sym3(const Sym3Args a, int nvb, const T* __restrict__ v,
+                                                 const T* __restrict__ x, size_t xs, const T* __restrict__ b,
+                                                 T* __restrict__ y, double* partial, unsigned* counter, double* dot) {
   dep_wait();
   static_assert(!DOT || K == 1, "fused dot: one right-hand side");
-  const int lane = (int)threadIdx.x % G;
+  __shared__ T sh[W][3 * K][32];
+  const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
   double part = 0.0;
   for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-    const SymRow R = sym3_locate<G>(a, vb);
+    const SymRow R = sym3_locate(a, vb, kSymRows, lane);
     T acc[3 * K];
 #pragma unroll
     for (int r = 0; r < 3 * K; ++r) acc[r] = T(0);
-    if (R.valid) sym3_row<G, U, K, T>(a, R, lane, v, x, xs, acc);
+    if (R.valid) sym3_row<W, U, K, T>(a, R, w, v, x, xs, acc);
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1)
+    for (int r = 0; r < 3 * K; ++r) sh[w][r][lane] = acc[r];
+    __syncthreads();
+    for (int r = w; r < 3 * K; r += W) {
+      T s[W];
 #pragma unroll
-      for (int r = 0; r < 3 * K; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
-    if (R.valid && lane == 0) {
+      for (int u = 0; u < W; ++u) s[u] = sh[u][r][lane];
 #pragma unroll
-      for (int r = 0; r < 3 * K; ++r) {
+      for (int o = W / 2; o; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < o; ++u) s[u] += s[u + o];
+      if (R.valid) {
         const size_t i = r * xs + R.row;
-        y[i] = b ? b[i] - acc[r] : acc[r];
-        if (DOT) part += (double)(acc[r] * x[i]);
+        y[i] = b ? b[i] - s[0] : s[0];
+        if (DOT) part += (double)(s[0] * x[i]);
       }
     }
+    __syncthreads();
   }
   if (DOT) grid_sum(part, partial, counter, dot);
 }
@@ -232,20 +233,21 @@ __global__ void __launch_bounds__(kSymBlock) k_sym3(const Sym3Args a, int nvb, c
 // y = b - A x in double-float arithmetic: A = vh + vl, x = xh + xl (FP32
 // pairs); K right-hand sides (x, b, y: 3K component-major components), each
 // stored block read once for all K
-template <int G, int K = 1>
-__global__ void __launch_bounds__(kSymBlock) k_sym3_df(const Sym3Args a, const float* __restrict__ vh,
+template <int W, int U, int K>
+__global__ void __launch_bounds__(32 * W) k_sym3_df(const Sym3Args a, const float* __restrict__ vh,
                                                       const float* __restrict__ vl, const float* __restrict__ xh,
                                                       const float* __restrict__ xl, size_t xs,
                                                       const double* __restrict__ b, double* __restrict__ y) {
   dep_wait();
-  const SymRow R = sym3_locate<G>(a, (int)blockIdx.x);
-  const int lane = (int)threadIdx.x % G;
+  constexpr int G = W;
+  __shared__ DF sh[W][3 * K][32];
+  const int lane = (int)threadIdx.x >> 5, slot = (int)threadIdx.x & 31;  // (lane: the warp, as in sym3_row)
+  const SymRow R = sym3_locate(a, (int)blockIdx.x, kSymRows, slot);
   const int c = R.c;
   const int last = (int)xs - 1;
   DF acc[3 * K];
 #pragma unroll
   for (int r = 0; r < 3 * K; ++r) acc[r] = DF{0.f, 0.f};
-  constexpr int U = K > 1 ? 1 : (SymBatch<G>::U > 4 ? 4 : SymBatch<G>::U);
   if (R.valid) {
     const size_t rc = (size_t)a.prows[c];
     const int u0 = a.ubeg[c], nu = a.ubeg[c + 1] - u0;
@@ -318,18 +320,15 @@ __global__ void __launch_bounds__(kSymBlock) k_sym3_df(const Sym3Args a, const f
     }
   }
 #pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1)
+  for (int r = 0; r < 3 * K; ++r) sh[lane][r][slot] = acc[r];
+  __syncthreads();
+  for (int r = lane; r < 3 * K; r += W) {
+    DF s = sh[0][r][slot];
 #pragma unroll
-    for (int r = 0; r < 3 * K; ++r) {
-      const float oh = __shfl_xor_sync(0xffffffffu, acc[r].h, o);
-      const float ol = __shfl_xor_sync(0xffffffffu, acc[r].l, o);
-      df_add(acc[r], oh, ol);
-    }
-  if (R.valid && lane == 0) {
-#pragma unroll
-    for (int r = 0; r < 3 * K; ++r) {
+    for (int u = 1; u < W; ++u) df_add(s, sh[u][r][slot].h, sh[u][r][slot].l);
+    if (R.valid) {
       const size_t i = r * xs + R.row;
-      y[i] = b[i] - ((double)acc[r].h + (double)acc[r].l);
+      y[i] = b[i] - ((double)s.h + (double)s.l);
     }
   }
 }
@@ -340,98 +339,88 @@ double sym3_bytes(const Sym3Op& so, int esz, int rows, int streams) {
   return (double)so.total * esz + (double)esz * 3.0 * rows * (1 + streams);
 }
 
-template <int G, int U>
-static void sym3_launch_g(const Exec& ex, const Csr& m, const double* x, double* y, const double* b,
-                          const DotScratch* ds, double* dot) {
-  const Sym3Op& so = *m.sym;
-  const Sym3Args a = sym3_args(so, G);
-  const int nvb = sym3_blocks(so, a);
-  if (nvb == 0) return;
-  // one resident wave walks the virtual blocks in plane order (measured faster
-  // than one block per virtual block: 171 against 200 us at 48^3)
-  static thread_local int wave[2] = {};  // resident blocks per variant (dot or not)
-  int& w = wave[dot ? 1 : 0];
+// one resident wave of a kernel walks the virtual blocks in plane order
+template <class F> static int sym3_wave(F kernel, int block, int& w) {
   if (!w) {
     int dev = 0, sms = 0, occ = 0;
     SK_CUDA(cudaGetDevice(&dev));
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (dot) SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, double, true>, kSymBlock, 0));
-    else SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<G, U, double, false>, kSymBlock, 0));
+    SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, block, 0));
     w = std::max(1, sms * std::max(1, occ));
   }
-  const int grid = std::min(nvb, w);
+  return w;
+}
+
+template <int W, int U>
+static void sym3_launch_w(const Exec& ex, const Csr& m, const double* x, double* y, const double* b,
+                          const DotScratch* ds, double* dot) {
+  const Sym3Op& so = *m.sym;
+  const Sym3Args a = sym3_args(so);
+  const int nvb = sym3_blocks(so, a);
+  if (nvb == 0) return;
+  static thread_local int wave[2] = {};  // resident blocks per variant (dot or not)
   if (dot) {
+    const int grid = std::min(nvb, sym3_wave(k_sym3<W, U, double, true>, 32 * W, wave[1]));
     SK_REQUIRE(ds && ds->fused_partial && grid <= ds->fused_cap, STOKES_ERR_ARG, "fused dot scratch too small");
-    launch_dep(k_sym3<G, U, double, true>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y,
-                                                    ds->fused_partial, ds->fused_counter, dot);
+    launch_dep(k_sym3<W, U, double, true>, grid, 32 * W, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y,
+               ds->fused_partial, ds->fused_counter, dot);
   } else {
-    launch_dep(k_sym3<G, U, double, false>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
-                                                     nullptr, nullptr);
+    const int grid = std::min(nvb, sym3_wave(k_sym3<W, U, double, false>, 32 * W, wave[0]));
+    launch_dep(k_sym3<W, U, double, false>, grid, 32 * W, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
+               nullptr, nullptr);
   }
-  SK_CHECK_LAUNCH();
 }
 
 // four right-hand sides (x, y, b: [4][3][rows]): every stored block read once
-// for the four; one thread per row, two entries' loads in flight
+// for the four
 void sym3_launch4(const Exec& ex, const Csr& m, const double* x, double* y, const double* b) {
   const Sym3Op& so = *m.sym;
-  const Sym3Args a = sym3_args(so, 1);
+  const Sym3Args a = sym3_args(so);
   const int nvb = sym3_blocks(so, a);
   if (nvb == 0) return;
-  static thread_local int w = 0;
-  if (!w) {
-    int dev = 0, sms = 0, occ = 0;
-    SK_CUDA(cudaGetDevice(&dev));
-    SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sym3<1, 2, double, false, 4>, kSymBlock, 0));
-    w = std::max(1, sms * std::max(1, occ));
-  }
-  const int grid = std::min(nvb, w);
-  launch_dep(k_sym3<1, 2, double, false, 4>, grid, kSymBlock, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
-                                                       nullptr, nullptr);
-  SK_CHECK_LAUNCH();
+  static thread_local int wave = 0;
+  const int grid = std::min(nvb, sym3_wave(k_sym3<4, 1, double, false, 4>, 128, wave));
+  launch_dep(k_sym3<4, 1, double, false, 4>, grid, 128, 0, ex, a, nvb, so.v64, x, (size_t)m.rows, b, y, nullptr,
+             nullptr, nullptr);
 }
+
+// Eight warps per 32 rows below 2^15 rows, four above: FP64 with the fused dot at
+// 8^3 16.7 us against 20.9 for four (a thread per row: 45), at 24^3 100 against
+// 104 for eight (148); the double-float residual at 48^3 298 us against 316 and
+// 374 for eight (one, two entries in flight) and 321 for a thread per row.
+constexpr int kSymWide = 1 << 15;
 
 void sym3_launch(const Exec& ex, const Csr& m, const double* x, double* y, const double* b, const DotScratch* ds,
                  double* dot) {
-  // (threads per row, entries in flight per lane)
-  const int g = m.sym->group, u = m.sym->batch;
-  if (g == 1 && u == 2) sym3_launch_g<1, 2>(ex, m, x, y, b, ds, dot);
-  else if (g == 1 && u == 4) sym3_launch_g<1, 4>(ex, m, x, y, b, ds, dot);
-  else if (g == 1) sym3_launch_g<1, 8>(ex, m, x, y, b, ds, dot);
-  else if (g == 2 && u == 2) sym3_launch_g<2, 2>(ex, m, x, y, b, ds, dot);
-  else if (g == 2) sym3_launch_g<2, 4>(ex, m, x, y, b, ds, dot);
-  else if (g == 4) sym3_launch_g<4, 2>(ex, m, x, y, b, ds, dot);
-  else sym3_launch_g<8, 1>(ex, m, x, y, b, ds, dot);
-}
-
-template <int G>
-static void sym3_df_g(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y) {
-  const Sym3Op& so = *m.sym;
-  const Sym3Args a = sym3_args(so, G);
-  const int grid = sym3_blocks(so, a);
-  if (grid == 0) return;
-  launch_dep(k_sym3_df<G>, grid, kSymBlock, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
-  SK_CHECK_LAUNCH();
-}
-
-// four right-hand sides in one sweep (one thread per row, one entry in flight)
-void sym3_residual_df4(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y) {
-  const Sym3Op& so = *m.sym;
-  const Sym3Args a = sym3_args(so, 1);
-  const int grid = sym3_blocks(so, a);
-  if (grid == 0) return;
-  launch_dep(k_sym3_df<1, 4>, grid, kSymBlock, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
-  SK_CHECK_LAUNCH();
+  // entries in flight per warp lane: sym_batch (2 by default)
+  const int u = m.sym->batch;
+  if (m.rows < kSymWide) {
+    if (u >= 4) sym3_launch_w<8, 4>(ex, m, x, y, b, ds, dot);
+    else sym3_launch_w<8, 2>(ex, m, x, y, b, ds, dot);
+  } else {
+    if (u >= 4) sym3_launch_w<4, 4>(ex, m, x, y, b, ds, dot);
+    else sym3_launch_w<4, 2>(ex, m, x, y, b, ds, dot);
+  }
 }
 
 void sym3_residual_df(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y) {
-  switch (m.sym->group) {
-    case 1: sym3_df_g<1>(ex, m, xh, xl, b, y); break;
-    case 2: sym3_df_g<2>(ex, m, xh, xl, b, y); break;
-    case 8: sym3_df_g<8>(ex, m, xh, xl, b, y); break;
-    default: sym3_df_g<4>(ex, m, xh, xl, b, y); break;
-  }
+  const Sym3Op& so = *m.sym;
+  const Sym3Args a = sym3_args(so);
+  const int grid = sym3_blocks(so, a);
+  if (grid == 0) return;
+  if (m.rows < kSymWide)
+    launch_dep(k_sym3_df<8, 2, 1>, grid, 256, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
+  else
+    launch_dep(k_sym3_df<4, 2, 1>, grid, 128, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
+}
+
+// four right-hand sides in one sweep (one entry in flight per lane)
+void sym3_residual_df4(const Exec& ex, const Csr& m, const float* xh, const float* xl, const double* b, double* y) {
+  const Sym3Op& so = *m.sym;
+  const Sym3Args a = sym3_args(so);
+  const int grid = sym3_blocks(so, a);
+  if (grid == 0) return;
+  launch_dep(k_sym3_df<4, 1, 4>, grid, 128, 0, ex, a, so.v32, so.v32lo, xh, xl, (size_t)m.rows, b, y);
 }
 
 }  // namespace sk
