@@ -10,6 +10,7 @@
 #include <map>
 #include <memory>
 #include <tuple>
+#include <type_traits>
 #include <stdexcept>
 #include <string>
 #include <unordered_map>
@@ -530,10 +531,10 @@ struct AssemblyOut {
   double* lumped = nullptr; // Lambda_V per interior node
   double* mv = nullptr;     // scalar P2 mass M on the P2P2 pattern
 };
-// Returns the number of inverted/degenerate tetrahedra.
-long long assemble(const Exec& ex, int n, const double* X, double mu, double dt,
-                   double eps, const Csr& p2, const Csr& p1, const Csr* b, const Csr* bt,
-                   const AssemblyOut& out, int* d_bad);
+// Adds the number of inverted or degenerate tetrahedra to *d_bad (device). No
+// host synchronisation.
+void assemble(const Exec& ex, int n, const double* X, double mu, double dt, double eps, const Csr& p2, const Csr& p1,
+              const Csr* b, const Csr* bt, const AssemblyOut& out, int* d_bad);
 // |K| per tetrahedron (index 6 * cube + p) of an n^3 Kuhn mesh
 void tet_volumes(const Exec& ex, int n, const double* X, double* vol);
 // F = M_V f from precomputed tet volumes (vol non-null; else as below)
@@ -662,16 +663,52 @@ struct DotScratch {
 };
 
 #ifdef __CUDACC__
-// Deterministic sum over the grid of one double per thread; every thread of
+__device__ __forceinline__ DF df_warp_sum(DF s) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const float h = __shfl_down_sync(0xffffffffu, s.h, o), l = __shfl_down_sync(0xffffffffu, s.l, o);
+    df_add(s, h, l);
+  }
+  return s;
+}
+// K sums over a warp's lanes by halving exchanges (K adds per lane instead of 5 K:
+// an FP64 add holds an SM's few FP64 lanes for 16 clocks); lanes whose low bits
+// are 0 end up with sum warp_sums_index<K>(lane) in v[0]
+template <int K> __device__ __forceinline__ void warp_sums(double (&v)[K], int lane) {
+#pragma unroll
+  for (int o = 16, cnt = K; o; o >>= 1) {
+    if (cnt > 1) {
+      cnt >>= 1;
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < cnt; ++i) {
+        const double send = up ? v[i] : v[i + cnt], keep = up ? v[i + cnt] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+}
+template <int K> __device__ __forceinline__ int warp_sums_index(int lane) { return lane / (32 / K); }
+// Deterministic sum over the grid of one value per thread; every thread of
 // every block must call it (no early return before). Warp shuffles, then the
 // warps of a block in order, give partial[blockIdx.x]; the last block to
 // finish adds the partials in block order, writes *out and resets *counter.
-__device__ __forceinline__ void grid_sum(double v, double* partial, unsigned* counter, double* out) {
+// With a double-float value (products of FP32 vectors that used to be rounded to
+// FP32 first) the warps sum on the FP32 units.
+template <class V>
+__device__ __forceinline__ void grid_sum(V v, double* partial, unsigned* counter, double* out) {
   __shared__ double sh_[32];
   __shared__ bool last_;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if (lane == 0) sh_[wid] = v;
+  if constexpr (std::is_same<V, DF>::value) {
+    v = df_warp_sum(v);
+    if (lane == 0) sh_[wid] = (double)v.h + (double)v.l;
+  } else {
+    for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) sh_[wid] = v;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
