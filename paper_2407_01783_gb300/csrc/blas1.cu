@@ -35,7 +35,6 @@ template <class T> struct DotArgs {
   const T* x[kMaxDots];
   const T* y[kMaxDots];
   int k;
-  int compensated;  // FP32 inputs: per-thread Neumaier sums in FP32, FP64 across threads
   size_t n;
   double* partial;
   unsigned* counter;
@@ -49,47 +48,7 @@ __global__ void __launch_bounds__(256) k_dots(DotArgs<T> a) {
 #pragma unroll
   for (int j = 0; j < K; ++j) s[j] = 0.0;
   size_t stride = (size_t)gridDim.x * blockDim.x;
-  if (a.compensated) {
-    // GB300 runs FP64 at a small fraction of its FP32 rate, so products and
-    // per-thread sums of FP32 vectors stay in FP32 with Neumaier's compensated
-    // summation (error ~ eps_32 per product, not per partial sum); only the
-    // cross-thread reduction is FP64.
-    // four independent accumulators per dot keep four loads per vector in
-    // flight per thread
-    float fs[K][4], fc[K][4];
-#pragma unroll
-    for (int j = 0; j < K; ++j)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) fs[j][u] = 0.f, fc[j][u] = 0.f;
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 3 * stride < a.n; i += 4 * stride) {
-#pragma unroll
-      for (int j = 0; j < K; ++j) {
-        float p[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) p[u] = (float)a.x[j][i + u * stride] * (a.y[j] ? (float)a.y[j][i + u * stride] : 1.f);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float t = fs[j][u] + p[u];
-          fc[j][u] += fabsf(fs[j][u]) >= fabsf(p[u]) ? (fs[j][u] - t) + p[u] : (p[u] - t) + fs[j][u];
-          fs[j][u] = t;
-        }
-      }
-    }
-    for (; i < a.n; i += stride) {
-#pragma unroll
-      for (int j = 0; j < K; ++j) {
-        const float p = (float)a.x[j][i] * (a.y[j] ? (float)a.y[j][i] : 1.f);
-        const float t = fs[j][0] + p;
-        fc[j][0] += fabsf(fs[j][0]) >= fabsf(p) ? (fs[j][0] - t) + p : (p - t) + fs[j][0];
-        fs[j][0] = t;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < K; ++j)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s[j] += (double)fs[j][u] + (double)fc[j][u];
-  } else {
+  {
     double t[K][4];
 #pragma unroll
     for (int j = 0; j < K; ++j)
@@ -147,17 +106,84 @@ __global__ void __launch_bounds__(256) k_dots(DotArgs<T> a) {
   if (threadIdx.x == 0) *a.counter = 0u;
 }
 
+// out = x . y (y null: sum of x) of FP32 vectors in double-float arithmetic from
+// the products (exact, df_dot) to the sum over the grid, in a fixed order: no
+// FP64 operations, whose few units bounded the reduction of short vectors.
+// blockDim.x = 1024 always; a single block (vectors up to kDotOneBlock) needs
+// no partials and no counter.
+// sum over a block of 32 warps, valid in thread 0; sh: 32 entries
+__device__ __forceinline__ DF df_block_sum(DF s, DF* sh) {
+  s = df_warp_sum(s);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x < 32) s = df_warp_sum(sh[threadIdx.x]);
+  return s;
+}
+__global__ void __launch_bounds__(1024) k_dot_df(size_t n, const float* __restrict__ x, const float* __restrict__ y,
+                                                double* partial, unsigned* counter, double* out) {
+  dep_wait();
+  __shared__ DF sh[32];
+  __shared__ bool last;
+  DF s[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  const size_t stride = (size_t)gridDim.x * 1024;
+  size_t i = (size_t)blockIdx.x * 1024 + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    float a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] = x[i + u * stride], b[u] = y ? y[i + u * stride] : 1.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) df_dot(s[u & 1], a[u], b[u]);
+  }
+  for (; i < n; i += stride) df_dot(s[0], x[i], y ? y[i] : 1.f);
+  df_add(s[0], s[1].h, s[1].l);
+  DF t = df_block_sum(s[0], sh);
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0) *out = (double)t.h + (double)t.l;
+    return;
+  }
+  if (threadIdx.x == 0) {
+    reinterpret_cast<DF*>(partial)[blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  t = DF{0.f, 0.f};
+  if (threadIdx.x < gridDim.x) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(partial) + threadIdx.x);
+    t = DF{v.x, v.y};
+  }
+  t = df_block_sum(t, sh);
+  if (threadIdx.x == 0) {
+    *out = (double)t.h + (double)t.l;
+    *counter = 0u;
+  }
+}
+// Whole solves with the line at 0, 2^14, 2^17 entries (ms): 12^3 16.8, 16.4,
+// 17.0; 33^3 64.9, 64.9, 66.6; 48^3 100.2, 99.9, 104.5. Mean over a solve's dots,
+// with compensated FP32 sums and an FP64 reduction before: 12^3 5.2 -> 3.1 us,
+// 48^3 11.5 -> 5.1 us.
+constexpr size_t kDotOneBlock = (size_t)1 << 14;
+
 template <class T>
 void dots(const Exec& ex, const DotScratch& ds, int k, const T* const* x, const T* const* y, size_t n, double* out,
           int mode) {
   SK_REQUIRE(k >= 1 && k <= kMaxDots, STOKES_ERR_ARG, "dots: bad count");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, 0.0 + (double)sizeof(T) * n * (2.0 * k));
+  if constexpr (std::is_same<T, float>::value) {
+    if (mode == kDotFast || (mode == kDotAuto && n >= kDoubleFloatMin)) {
+      const int grid = n <= kDotOneBlock ? 1 : (int)std::min<long long>(152, cdiv((long long)n, 1024));
+      for (int j = 0; j < k; ++j)
+        launch_dep(k_dot_df, grid, 1024, 0, ex, n, x[j], y ? y[j] : (const float*)nullptr, ds.partial, ds.counter,
+                   out + j);
+      return;
+    }
+  }
   DotArgs<T> a{};
   for (int j = 0; j < k; ++j) a.x[j] = x[j], a.y[j] = y ? y[j] : nullptr;
   a.k = k;
   a.n = n;
-  a.compensated = std::is_same<T, float>::value &&
-                  (mode == kDotFast || (mode == kDotAuto && n >= kCompensatedMin));
   a.partial = ds.partial;
   a.counter = ds.counter;
   a.out = out;
@@ -195,40 +221,33 @@ template <class T> struct MultiArgs {
 template <class T, int K>
 __global__ void __launch_bounds__(256) k_mdot(MultiArgs<T> a) {
   dep_wait();
-  double s[K];
-  if constexpr (std::is_same<T, float>::value) {
-    // FP32 vectors: per-thread double-float sums (df_dot) on the FP32 units
-    // (FP64 arithmetic would bound the kernel before memory does)
-    DF d[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) d[i] = DF{0.f, 0.f};
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.n; e += (size_t)gridDim.x * blockDim.x) {
-      const float we = a.wr[e];
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < a.k) df_dot(d[i], a.v[i][e], we);
-    }
-#pragma unroll
-    for (int i = 0; i < K; ++i) s[i] = (double)d[i].h + (double)d[i].l;
-  } else {
-#pragma unroll
-    for (int i = 0; i < K; ++i) s[i] = 0.0;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.n; e += (size_t)gridDim.x * blockDim.x) {
-      const double we = (double)a.wr[e];
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < a.k) s[i] += (double)a.v[i][e] * we;
-    }
-  }
   __shared__ double sh[8][K];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  using S = typename std::conditional<std::is_same<T, float>::value, DF, double>::type;
+  S d[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) d[i] = S{};
+#pragma unroll(K <= 8 ? 2 : 1)
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.n; e += (size_t)gridDim.x * blockDim.x) {
+    const T we = a.wr[e];
+    T v[K];  // all loads of an element before the first use
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = i < a.k ? a.v[i][e] : T(0);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      if constexpr (std::is_same<T, float>::value) df_dot(d[i], v[i], we);  // (on the FP32 units)
+      else d[i] += v[i] * we;
+    }
+  }
+  double acc[K];
 #pragma unroll
   for (int i = 0; i < K; ++i) {
-    double v = s[i];
-    for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[wid][i] = v;
+    if constexpr (std::is_same<T, float>::value) acc[i] = (double)d[i].h + (double)d[i].l;
+    else acc[i] = d[i];
   }
+  warp_sums<K>(acc, lane);
+  if (lane % (32 / K) == 0) sh[wid][warp_sums_index<K>(lane)] = acc[0];
   __syncthreads();
   if (threadIdx.x < a.k) {
     double v = 0.0;
@@ -259,10 +278,11 @@ __global__ void __launch_bounds__(256) k_maxpy(MultiArgs<T> a) {
   if (threadIdx.x < K) h[threadIdx.x] = threadIdx.x < a.k ? (T)(a.sign * (a.dev ? a.dev[threadIdx.x] : a.c[threadIdx.x])) : T(0);
   __syncthreads();
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.n; e += (size_t)gridDim.x * blockDim.x) {
-    T acc = a.w[e];
+    T acc = a.w[e], v[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i)
-      if (i < a.k) acc += h[i] * a.v[i][e];
+    for (int i = 0; i < K; ++i) v[i] = i < a.k ? a.v[i][e] : T(0);  // all loads before the first use
+#pragma unroll
+    for (int i = 0; i < K; ++i) acc += h[i] * v[i];
     a.w[e] = acc;
   }
 }
@@ -273,10 +293,12 @@ static inline int pow2_at_least(int k) {
   return K;
 }
 
+constexpr int kMdotBlocks = 2 * 152;
 template <class T>
 void mdot(const Exec& ex, const DotScratch& ds, int k, const T* const* V, const T* w, size_t n, double* out) {
   SK_REQUIRE(k >= 1 && k <= kMaxBasis, STOKES_ERR_ARG, "mdot: bad count");
-  const int grid = (int)std::min<long long>(kDotBlocks, std::max<long long>(1, cdiv((long long)n, 256)));
+  // few blocks per SM: each warp ends with about 4 k FP64 operations
+  const int grid = (int)std::min<long long>(kMdotBlocks, std::max<long long>(1, cdiv((long long)n, 256)));
   SK_REQUIRE(ds.fused_partial && (long long)grid * k <= ds.fused_cap, STOKES_ERR_ARG, "mdot: scratch too small");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * n * (k + 1.0));
   MultiArgs<T> a{};
@@ -390,7 +412,7 @@ template <class T> void cg_update(const Exec& ex, size_t n, Coef a, const T* d, 
 }
 
 // x += a d; r -= a q; *rr = r . r (new r), the squares summed per thread in
-// FP64 and over the grid in a fixed order (grid_sum)
+// FP64 (FP64 vectors) or double-float and over the grid in a fixed order
 template <class T>
 __global__ void k_cg_update_rr(size_t n, Coef a, const T* __restrict__ d, T* __restrict__ x, const T* __restrict__ q,
                                T* __restrict__ r, int* flag, double* partial, unsigned* counter, double* rr) {
@@ -400,12 +422,14 @@ __global__ void k_cg_update_rr(size_t n, Coef a, const T* __restrict__ d, T* __r
   if (blockIdx.x == 0 && threadIdx.x == 0 && flag && a.den && !(*a.den > 0.0))
     atomicOr(flag, 1);  // p^T A p <= 0: breakdown
   const T av = (T)ad;
-  double s = 0.0;
+  using S = typename std::conditional<std::is_same<T, float>::value, DF, double>::type;
+  S s = S{};
   SK_LOOP(i) {
     x[i] += av * d[i];
     const T rn = r[i] - av * q[i];
     r[i] = rn;
-    s += (double)(rn * rn);
+    if constexpr (std::is_same<T, float>::value) df_dot(s, rn, rn);
+    else s += rn * rn;
   }
   grid_sum(s, partial, counter, rr);
 }

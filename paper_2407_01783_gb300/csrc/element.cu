@@ -366,8 +366,7 @@ __global__ void __launch_bounds__(256) k_el_sum(int n, int nb, const float* __re
     }
   }
   if (DOT)
-    grid_sum((double)o.s.h + (double)o.s.l, partial + (size_t)blockIdx.y * gridDim.x, counter + blockIdx.y,
-             dot + blockIdx.y);
+    grid_sum(o.s, partial + (size_t)blockIdx.y * gridDim.x, counter + blockIdx.y, dot + blockIdx.y);
 }
 
 size_t element_part_words(int n) { return el_part_words((size_t)n * n * n); }

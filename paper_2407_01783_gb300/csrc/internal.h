@@ -769,10 +769,10 @@ double sym3_bytes(const Sym3Op& so, int esz, int rows, int streams);
 int sym3_grid(const Sym3Op& so);
 // most blocks of one dot-fused BSR3 product launch (fused-dot partial capacity)
 int bsr3_dot_grid(const Csr& m);
-// FP32 vectors at least this long use compensated FP32 per-thread sums in
-// dots() (velocity-sized vectors of the inner solves); shorter ones
-// (pressure-sized, the outer Schur iteration) accumulate in FP64 throughout.
-constexpr size_t kCompensatedMin = (size_t)1 << 20;
+// FP32 vectors at least this long are summed in double-float arithmetic by dots()
+// (velocity-sized vectors of the inner solves); shorter ones (pressure-sized, the
+// outer Schur iteration) accumulate in FP64 throughout.
+constexpr size_t kDoubleFloatMin = (size_t)1 << 20;
 // Rows below which the stencil kernels spread a row's entries over 8, 4 and 2
 // warps (k_stencil_w): FP32 component-major, FP64, interleaved. Whole solves in
 // ms with the lines (powers of two) set to ...: FP32, 48^3: {14, 16, 18} 102.5,
@@ -786,9 +786,9 @@ constexpr long long kStencilSplit32[3] = {1 << 15, 1 << 16, 1 << 19};
 constexpr long long kStencilSplit64[3] = {1 << 15, 1 << 17, 1 << 18};
 constexpr long long kStencilSplitIL[3] = {1 << 16, 1 << 18, 1 << 18};
 // out[i] = sum_j x_i[j] * y_i[j] for i < k (y_i == nullptr means all ones).
-// Accumulation of FP32 dot products: kDotAuto = compensated FP32 partial sums
-// for vectors of at least kCompensatedMin entries, kDotFast = compensated for
-// any length (inner solves), kDotExact = FP64 throughout (outer Krylov).
+// Accumulation of FP32 dot products: kDotAuto = double-float for vectors of at
+// least kDoubleFloatMin entries, kDotFast = double-float for any length (inner
+// solves), kDotExact = FP64 throughout (outer Krylov).
 enum { kDotAuto = 0, kDotFast = 1, kDotExact = 2 };
 template <class T> void dots(const Exec& ex, const DotScratch& ds, int k, const T* const* x,
                              const T* const* y, size_t n, double* out, int mode = kDotAuto);

@@ -40,21 +40,21 @@ __global__ void __launch_bounds__(256) k_kdot(KSeg s, const T* __restrict__ x, c
   dep_wait();
   const int k = blockIdx.y;
   const size_t n = s.len();
-  double t = 0.0;
   if constexpr (std::is_same<T, float>::value) {
     DF a{0.f, 0.f};
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
       const size_t i = s.at(k, e);
       df_dot(a, x[i], y ? y[i] : 1.f);
     }
-    t = (double)a.h + (double)a.l;
+    grid_sum((double)a.h + (double)a.l, partial + (size_t)k * gridDim.x, counter + k, out + k);
   } else {
+    double t = 0.0;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
       const size_t i = s.at(k, e);
       t += (double)x[i] * (y ? (double)y[i] : 1.0);
     }
+    grid_sum(t, partial + (size_t)k * gridDim.x, counter + k, out + k);
   }
-  grid_sum(t, partial + (size_t)k * gridDim.x, counter + k, out + k);
 }
 
 // y_k = a_k x_k + b_k y_k on the chosen segment (x may alias y)
@@ -74,6 +74,34 @@ __global__ void __launch_bounds__(256) k_kaxpby(KSeg s, KCoefs a, const T* x, KC
     const size_t i = s.at(k, e);
     y[i] = bv == T(0) ? av * x[i] : av * x[i] + bv * y[i];
   }
+}
+
+// one CG update of K plain blocks: x_k += a_k d_k, r_k -= a_k q_k and, with rr,
+// rr[k] = r_k . r_k of the new residual (per-thread sums as k_kdot)
+template <class T>
+__global__ void __launch_bounds__(256) k_kcg_update(size_t n, KCoefs a, const T* __restrict__ d, T* __restrict__ x,
+                                                    const T* __restrict__ q, T* __restrict__ r, int* flag,
+                                                    double* partial, unsigned* counter, double* rr) {
+  dep_wait();
+  const int k = blockIdx.y;
+  __shared__ double av_;
+  if (threadIdx.x == 0) av_ = a.value(k, blockIdx.x == 0 ? flag : nullptr);
+  __syncthreads();
+  const T av = (T)av_;
+  using S = typename std::conditional<std::is_same<T, float>::value, DF, double>::type;
+  S s = S{};
+  const size_t off = (size_t)k * n;
+#pragma unroll 2
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t i = off + e;
+    x[i] += av * d[i];
+    const T rn = r[i] - av * q[i];
+    r[i] = rn;
+    if constexpr (std::is_same<T, float>::value) df_dot(s, rn, rn);
+    else s += rn * rn;
+  }
+  if (!rr) return;
+  grid_sum(s, partial + (size_t)k * gridDim.x, counter + k, rr + k);
 }
 
 // y_k += c_k (a constant per right-hand side, c_k = scale * num_k / den_k)
@@ -98,40 +126,34 @@ __global__ void __launch_bounds__(256) k_kmdot(KSeg s, KBasis<T> V, int J, const
   dep_wait();
   const int k = blockIdx.y;
   const size_t n = s.len();
-  double acc[KB];
-  if constexpr (std::is_same<T, float>::value) {  // double-float per thread, as k_kdot
-    DF a[KB];
-#pragma unroll
-    for (int i = 0; i < KB; ++i) a[i] = DF{0.f, 0.f};
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-      const size_t q = s.at(k, e);
-      const float we = w[q];
-#pragma unroll
-      for (int i = 0; i < KB; ++i)
-        if (i < J) df_dot(a[i], V.v[i][q], we);
-    }
-#pragma unroll
-    for (int i = 0; i < KB; ++i) acc[i] = (double)a[i].h + (double)a[i].l;
-  } else {
-#pragma unroll
-    for (int i = 0; i < KB; ++i) acc[i] = 0.0;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-      const size_t a = s.at(k, e);
-      const double we = (double)w[a];
-#pragma unroll
-      for (int i = 0; i < KB; ++i)
-        if (i < J) acc[i] += (double)V.v[i][a] * we;
-    }
-  }
   __shared__ double sh[8][KB];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  using S = typename std::conditional<std::is_same<T, float>::value, DF, double>::type;  // as k_kdot
+  S d[KB];
+#pragma unroll
+  for (int i = 0; i < KB; ++i) d[i] = S{};
+#pragma unroll(KB <= 8 ? 2 : 1)
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t q = s.at(k, e);
+    const T we = w[q];
+    T v[KB];  // all loads of an element before the first use
+#pragma unroll
+    for (int i = 0; i < KB; ++i) v[i] = i < J ? V.v[i][q] : T(0);
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      if constexpr (std::is_same<T, float>::value) df_dot(d[i], v[i], we);
+      else d[i] += v[i] * we;
+    }
+  }
+  double acc[KB];
 #pragma unroll
   for (int i = 0; i < KB; ++i) {
-    double v = acc[i];
-    for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[wid][i] = v;
+    if constexpr (std::is_same<T, float>::value) acc[i] = (double)d[i].h + (double)d[i].l;
+    else acc[i] = d[i];
   }
+  warp_sums<KB>(acc, lane);
+  if (lane % (32 / KB) == 0) sh[wid][warp_sums_index<KB>(lane)] = acc[0];
   __syncthreads();
   double* part = partial + (size_t)k * KB * gridDim.x;
   if (threadIdx.x < J) {
@@ -169,10 +191,11 @@ __global__ void __launch_bounds__(256) k_kmaxpy(KSeg s, KBasis<T> V, int J, cons
   const size_t n = s.len();
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     const size_t a = s.at(k, e);
-    T acc = w[a];
+    T acc = w[a], v[KB];
 #pragma unroll
-    for (int i = 0; i < KB; ++i)
-      if (i < J) acc += c[i] * V.v[i][a];
+    for (int i = 0; i < KB; ++i) v[i] = i < J ? V.v[i][a] : T(0);  // all loads before the first use
+#pragma unroll
+    for (int i = 0; i < KB; ++i) acc += c[i] * v[i];
     w[a] = acc;
   }
 }
@@ -223,6 +246,16 @@ void kaxpby(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs
 }
 
 template <class T>
+void kcg_update(const Exec& ex, const DotScratch& ds, size_t n, int K, const KCoefs& a, const T* d, T* x, const T* q,
+                T* r, double* rr) {
+  if (!n) return;
+  const int gx = kgrid(n);
+  SK_REQUIRE(!rr || (long long)gx * K <= ds.k_cap, STOKES_ERR_ARG, "K-dot scratch too small");
+  ProfScope ps(ex, STOKES_KERNEL_BLAS1, 6.0 * sizeof(T) * n * K);
+  launch_dep(k_kcg_update<T>, dim3(gx, K), 256, 0, ex, n, a, d, x, q, r, ex.flag, ds.k_partial, ds.k_counter, rr);
+}
+
+template <class T>
 void kaddconst(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs& c, T* y) {
   SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kaddconst: 1 to 8 right-hand sides");
   const size_t len = seglen(nu, np, parts);
@@ -236,7 +269,8 @@ void kmdot(const Exec& ex, const DotScratch& ds, size_t nu, size_t np, int K, in
            double* out, int ld) {
   SK_REQUIRE(J >= 1 && J <= kMaxBasisK && K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kmdot: bad count");
   const size_t len = seglen(nu, np, 3);
-  const int gx = kgrid(len);
+  // few blocks per SM over all right-hand sides: each warp ends with about 4 J FP64 operations
+  const int gx = std::min(kgrid(len), std::max(1, 2 * kKGridMax / K));
   const int KB = pow2_ge(J);
   SK_REQUIRE(ds.k_partial && (long long)gx * K * KB <= ds.k_cap, STOKES_ERR_ARG, "kmdot: scratch too small");
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)sizeof(T) * K * len * (J + 1.0));
@@ -291,6 +325,8 @@ void ksub(const Exec& ex, int K, double* out, const double* a, const double* b) 
 #define SK_INSTK(T)                                                                                                  \
   template void kdot<T>(const Exec&, const DotScratch&, size_t, size_t, int, int, const T*, const T*, double*);     \
   template void kaxpby<T>(const Exec&, size_t, size_t, int, int, const KCoefs&, const T*, const KCoefs&, T*);      \
+  template void kcg_update<T>(const Exec&, const DotScratch&, size_t, int, const KCoefs&, const T*, T*, const T*,  \
+                              T*, double*);                                                                        \
   template void kaddconst<T>(const Exec&, size_t, size_t, int, int, const KCoefs&, T*);                           \
   template void kmdot<T>(const Exec&, const DotScratch&, size_t, size_t, int, int, const T* const*, const T*,      \
                          double*, int);                                                                              \

@@ -1312,14 +1312,11 @@ static int kpcg(stokes_ctx& c, size_t n, int K, Op&& op, Pre&& pre, const T* b, 
       op((const T*)d, (T*)q, D + 2 * K);
       ++it;
       KCoefs alpha = KCoefs::ratio(D + irz * K, D + 2 * K).mask(act);
-      KCoefs malpha = KCoefs::ratio(D + irz * K, D + 2 * K, -1.0).mask(act);
-      kaxpby<T>(c.ex, n, 0, K, 1, alpha, d, KCoefs::constant(1.0), x);
-      kaxpby<T>(c.ex, n, 0, K, 1, malpha, q, KCoefs::constant(1.0), r);
+      kcg_update<T>(c.ex, c.ds, n, K, alpha, d, x, q, r, fixed > 0 ? nullptr : D + 3 * K);
       if (fixed > 0) {
         if (it == cap) break;
         pre((const T*)r, (T*)z);
       } else {
-        kdot<T>(c.ex, c.ds, n, 0, K, 1, r, r, D + 3 * K);
         read_k_issue(c, D + 3 * K, s + 3 * K, K);
         pre((const T*)r, (T*)z);
         SK_CUDA(cudaEventSynchronize(c.ev_read));
