@@ -386,9 +386,14 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
   c.U_last = c.arena.alloc<double>(3 * (size_t)L0.nvi);
   c.P_last = c.arena.alloc<double>(L0.np);
   if (c.mixed) {
-    c.A.v32 = f32_copy(c, c.A.v64, 9 * (size_t)c.A.nnz);
-    c.A.v32lo = c.arena.alloc<float>(9 * (size_t)c.A.nnz);
-    to_f32_lo(c.ex, c.A.v64, c.A.v32, c.A.v32lo, 9 * (size_t)c.A.nnz);
+    // BSR3 copies only where a product reads them (14 GB at 96^3 otherwise): FP32
+    // products in formats 1 and 3, the velocity preconditioner A~_2, and the
+    // double-float residual without symmetric storage
+    if (!c.A.el || c.opt.vel_prec == 2) c.A.v32 = f32_copy(c, c.A.v64, 9 * (size_t)c.A.nnz);
+    if (!c.symA) {
+      c.A.v32lo = c.arena.alloc<float>(9 * (size_t)c.A.nnz);
+      to_f32_lo(c.ex, c.A.v64, c.A.v32, c.A.v32lo, 9 * (size_t)c.A.nnz);
+    }
     if (c.divB) {
       c.divB->v32 = f32_copy(c, c.divB->v64, 3 * (size_t)kDivS * L0.np);
     } else {
@@ -434,13 +439,14 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
       (k > 1 ? m.group4 : m.group) = g;
       return;
     }
+    if (m.st && m.rows >= m.st_min_single) return;  // its products read the stencil storage
     Csr probe = m;
     if (c.mixed && m.v32) probe.v64 = nullptr;
     autotune_group(c.ex, probe, nr, kind, k);
     m.group = probe.group;
     m.group4 = probe.group4;
   };
-  tune(c.A, 3, 1);
+  if (!c.A.sym_products) tune(c.A, 3, 1);
   if (c.A.sym) c.symA->batch = c.opt.sym_batch > 0 ? c.opt.sym_batch : 2;
   if (!c.divB) {
     tune(c.B, 1, 2);

@@ -1071,7 +1071,7 @@ static int read_flag(stokes_ctx& c) {
 static double full_residual(stokes_ctx& c, const double* F, const double* g, const double* U, const double* P,
                             double* rF, double* rg, double normFg) {
   const size_t nv = nvel(c), np = npres(c);
-  if (c.A.v32lo) {
+  if (c.mixed) {
     // mixed precision: the same FP64-accurate product on FP32 units
     Tmp<float> uh(c.pool, nv), ul(c.pool, nv);
     split_f64(c.ex, nv, U, uh, ul);
@@ -1712,7 +1712,7 @@ static void method2_k(stokes_ctx& c, int K, const T* R, T* X, const double* eta,
 static void full_residual_k(stokes_ctx& c, int K, const double* F, const double* g, const double* X, double* R,
                             const double* normFg, double* rel) {
   const size_t nv = nvel(c), np = npres(c), Kv = (size_t)K * nv;
-  if (K == 4 && c.A.v32lo && c.A.sym && c.A.sym->v32lo) {  // one sweep of each matrix for the four
+  if (K == 4 && c.A.sym && c.A.sym->v32lo) {  // one sweep of each matrix for the four
     Tmp<float> uh(c.pool, Kv), ul(c.pool, Kv);
     split_f64(c.ex, Kv, X, uh, ul);
     {
@@ -1726,7 +1726,7 @@ static void full_residual_k(stokes_ctx& c, int K, const double* F, const double*
    for (int k = 0; k < K; ++k) {
     const double* Uk = X + k * nv;
     double* rFk = R + k * nv;
-    if (c.A.v32lo) {
+    if (c.mixed) {
       Tmp<float> uh(c.pool, nv), ul(c.pool, nv);
       split_f64(c.ex, nv, Uk, uh, ul);
       bsr3_residual_df(c.ex, c.A, uh, ul, F + k * nv, rFk, STOKES_KERNEL_RESIDUAL);
@@ -2028,7 +2028,7 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       break;
     case STOKES_OP_LOAD: assemble_load(c.ex, c.n, c.lv[0].X, c.lv[0].A3, x, y, c.tet_vol); break;
     case STOKES_OP_A_DF: {
-      SK_REQUIRE(c.A.v32lo, STOKES_ERR_ARG, "double-float A needs a mixed-precision context");
+      SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "double-float A needs a mixed-precision context");
       Tmp<float> xh(c.pool, nv), xl(c.pool, nv);
       Tmp<double> zero_b(c.pool, nv);
       zero<double>(c, zero_b, nv);
