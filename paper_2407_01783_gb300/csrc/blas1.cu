@@ -216,6 +216,9 @@ template <class T> struct MultiArgs {
   double* out;
 };
 
+// All vectors' loads of an element are issued before the first is used, and the
+// lanes' sums end in halving exchanges. Up to 8 / 16 vectors at 33^3: 17 / 26 us
+// against 36 / 56 with a load at a time and five FP64 adds per warp and vector.
 // K: the compile-time bound (a power of two >= a.k), so the basis pointers and
 // accumulators are indexed statically
 template <class T, int K>

@@ -244,11 +244,12 @@ constexpr int kElBlock = 192;  // 32 cubes x 6 tetrahedra
 // 48^3), one thread per cube with 255 registers 35 us there and 8 us instead of
 // 3.4 us on small meshes (one long chain per cube). Product with k_el_sum
 // against the symmetric storage it replaced (2.8 TB/s on 446 MB at 48^3):
-// 8^3 7.8 us (12 us), 12^3 8 (16), 25^3 12 (31), 33^3 17 (60), 48^3 40 (165),
-// 64^3 87 (352), 96^3 350 (1267).
+// 12^3 7.6 us (16), 25^3 11 (31), 33^3 17 (60), 48^3 40 (165), 64^3 87 (352),
+// 96^3 289 (1267).
 // Error against FP64 over n = 2..96, mu dt from 1e-8 to 1e-2: N(0,1) vectors
-// 5.0e-8..7.0e-8 relative (the FP32 blocks: 6.3e-8..7.5e-8), smooth vectors
-// 5.0e-8..6.4e-6 (4.7e-8..1.9e-5).
+// 5.0e-8..7.0e-8 relative (the FP32 blocks: 6.3e-8..7.5e-8); smooth vectors
+// 6.4e-6 against 1.9e-5 where the stiffness dominates (96^3, mu = 1, dt = 1e-2),
+// 5.7e-8 against 4.8e-8 where the mass does (mu = dt = 1e-4).
 __global__ void __launch_bounds__(kElBlock, 4) k_el_strain(int n, const float* __restrict__ G, float mu,
                                                        const float* __restrict__ x, size_t xs,
                                                        float* __restrict__ part) {
