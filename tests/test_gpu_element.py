@@ -14,7 +14,7 @@ import workload as wl
 from oracle.assemble import StokesSystem
 from oracle.mesh import KuhnMesh
 
-from gpu_helpers import aos, cuda, gpu_module, host, soa
+from gpu_helpers import aos, cuda, gpu_module, host, soa, to_scipy
 
 pytestmark = pytest.mark.gpu
 
@@ -76,4 +76,23 @@ def test_fp32_transfers_without_matrices(n):
             size = host(S.apply(op, cuda(abs(x)), ny, level))  # (weights of both signs: a lower bound of |P||x|)
             got = host(S.apply(op + "_F32", cuda(x), ny, level))
             assert np.linalg.norm(got - want) <= BOUND * (np.linalg.norm(size) + np.linalg.norm(want))
+    S.close()
+
+
+@pytest.mark.parametrize("n", [3, 16, 17, 26, 33])
+def test_stencil_products_across_warp_splits(n):
+    """A~_3 and the P1 operators from stencil storage against their exported
+    CSR matrices, with level sizes on both sides of the lines where a row's
+    entries go over 8, 4, 2 warps or one thread (2^15, 2^17, 2^18 rows); sums
+    of up to 65 FP64 products."""
+    sk = gpu_module()
+    S = sk.Stokes(n, wl.kuhn_vertices(n, 0.16, 5), 1e-2, 1e-3)
+    rng = np.random.default_rng(n)
+    for op, comps in (("A3", 3), ("KQ", 1), ("MQ", 1), ("LQ", 1)):
+        rp, ci, v, shp = S.matrix(op)
+        M = to_scipy(rp, ci, v, shp)
+        x = rng.standard_normal((comps, shp[1]))
+        y = host(S.apply(op, cuda(x.ravel()), comps * shp[0])).reshape(comps, -1)
+        for c in range(comps):
+            assert np.linalg.norm(y[c] - M @ x[c]) <= 1e-14 * np.linalg.norm(abs(M) @ abs(x[c]))
     S.close()
