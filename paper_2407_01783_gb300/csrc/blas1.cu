@@ -616,28 +616,29 @@ void from_split(const Exec& ex, size_t rows, int nr, const T* src, T* dst, bool 
   split_launch<T, false>(ex, rows, nr, src, dst, il, sm);
 }
 
-template <class S, class D> __global__ void k_convert(size_t n, const S* __restrict__ x, D* __restrict__ y) {
+template <class S, class D> __global__ void k_convert(size_t n, S scale, const S* __restrict__ x, D* __restrict__ y) {
   dep_wait();
   SK_LOOP(i) {
-    y[i] = (D)x[i];
+    y[i] = (D)(scale * x[i]);
   }
 }
-template <class S, class D> void convert(const Exec& ex, size_t n, const S* x, D* y) {
+template <class S, class D> void convert(const Exec& ex, size_t n, const S* x, D* y, double scale) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + sizeof(D)) * n);
-  launch_dep(k_convert<S, D>, SK_GRID(n), n, x, y);
+  launch_dep(k_convert<S, D>, SK_GRID(n), n, (S)scale, x, y);
   SK_CHECK_LAUNCH();
 }
-template <class S, class D> __global__ void k_add_convert(size_t n, const S* __restrict__ x, D* __restrict__ y) {
+template <class S, class D>
+__global__ void k_add_convert(size_t n, D scale, const S* __restrict__ x, D* __restrict__ y) {
   dep_wait();
   SK_LOOP(i) {
-    y[i] += (D)x[i];
+    y[i] += scale * (D)x[i];
   }
 }
-template <class S, class D> void add_convert(const Exec& ex, size_t n, const S* x, D* y) {
+template <class S, class D> void add_convert(const Exec& ex, size_t n, const S* x, D* y, double scale) {
   if (!n) return;
   ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + 2 * sizeof(D)) * n);
-  launch_dep(k_add_convert<S, D>, SK_GRID(n), n, x, y);
+  launch_dep(k_add_convert<S, D>, SK_GRID(n), n, (D)scale, x, y);
   SK_CHECK_LAUNCH();
 }
 
@@ -735,10 +736,10 @@ void scalar_sub(const Exec& ex, double* out, const double* a, const double* b) {
   template void maxpy<T>(const Exec&, int, const double*, const double*, double, const T* const*, T*, size_t);
 SK_INST1(float)
 SK_INST1(double)
-template void convert<double, float>(const Exec&, size_t, const double*, float*);
-template void convert<float, double>(const Exec&, size_t, const float*, double*);
-template void convert<double, double>(const Exec&, size_t, const double*, double*);
-template void add_convert<float, double>(const Exec&, size_t, const float*, double*);
-template void add_convert<double, double>(const Exec&, size_t, const double*, double*);
+template void convert<double, float>(const Exec&, size_t, const double*, float*, double);
+template void convert<float, double>(const Exec&, size_t, const float*, double*, double);
+template void convert<double, double>(const Exec&, size_t, const double*, double*, double);
+template void add_convert<float, double>(const Exec&, size_t, const float*, double*, double);
+template void add_convert<double, double>(const Exec&, size_t, const double*, double*, double);
 
 }  // namespace sk

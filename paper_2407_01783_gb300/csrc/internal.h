@@ -823,10 +823,11 @@ template <class T> void cheb_first_il(const Exec& ex, size_t n, int nr, const T*
 // component-major [nr][rows] <-> node-interleaved [rows][nr] (nr = 4 or 12)
 template <class T> void to_interleaved(const Exec& ex, size_t rows, int nr, const T* cm, T* il);
 template <class T> void to_component_major(const Exec& ex, size_t rows, int nr, const T* il, T* cm);
-template <class S, class D> void convert(const Exec& ex, size_t n, const S* x, D* y);
+// y = scale x, y += scale x between precisions
+template <class S, class D> void convert(const Exec& ex, size_t n, const S* x, D* y, double scale = 1.0);
 // hi = FP32(x), lo = FP32(x - hi)
 void split_f64(const Exec& ex, size_t n, const double* x, float* hi, float* lo);
-template <class S, class D> void add_convert(const Exec& ex, size_t n, const S* x, D* y);
+template <class S, class D> void add_convert(const Exec& ex, size_t n, const S* x, D* y, double scale = 1.0);
 
 // ---------------------------------------------------------------------------
 // K right-hand sides in lockstep (multi.cu). A K-vector stores K systems'
@@ -903,6 +904,11 @@ template <class T> void kdot(const Exec& ex, const DotScratch& ds, size_t nu, si
 // y_k = a_k x_k + b_k y_k over the segment
 template <class T> void kaxpby(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs& a, const T* x,
                                const KCoefs& b, T* y);
+// y_k = a_k x_k, y_k += a_k x_k over whole segments (parts = 3), between precisions
+template <class S, class D>
+void kconvert(const Exec& ex, size_t nu, size_t np, int K, const KCoefs& a, const S* x, D* y);
+template <class S, class D>
+void kadd_convert(const Exec& ex, size_t nu, size_t np, int K, const KCoefs& a, const S* x, D* y);
 // one CG update of K plain blocks of length n: x_k += a_k d_k, r_k -= a_k q_k
 // and, with rr, rr[k] = r_k . r_k
 template <class T>

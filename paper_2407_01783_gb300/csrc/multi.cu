@@ -76,6 +76,20 @@ __global__ void __launch_bounds__(256) k_kaxpby(KSeg s, KCoefs a, const T* x, KC
   }
 }
 
+// y_k = a_k x_k or, with ADD, y_k += a_k x_k, between precisions (multiplied in FP64)
+template <class S, class D, bool ADD>
+__global__ void __launch_bounds__(256) k_kconvert(KSeg s, KCoefs a, const S* __restrict__ x, D* __restrict__ y) {
+  dep_wait();
+  const int k = blockIdx.y;
+  const double av = a.c[k];
+  const size_t n = s.len();
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t i = s.at(k, e);
+    const D v = (D)(av * (double)x[i]);
+    y[i] = ADD ? y[i] + v : v;
+  }
+}
+
 // one CG update of K plain blocks: x_k += a_k d_k, r_k -= a_k q_k and, with rr,
 // rr[k] = r_k . r_k of the new residual: one launch and six streams instead of
 // three launches and eight (means over a solve of six systems at 25^3: 13 us
@@ -250,6 +264,21 @@ void kaxpby(const Exec& ex, size_t nu, size_t np, int K, int parts, const KCoefs
   SK_CHECK_LAUNCH();
 }
 
+template <class S, class D>
+void kconvert(const Exec& ex, size_t nu, size_t np, int K, const KCoefs& a, const S* x, D* y) {
+  SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kconvert: 1 to 8 right-hand sides");
+  const size_t len = seglen(nu, np, 3);
+  ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + sizeof(D)) * K * len);
+  launch_dep(k_kconvert<S, D, false>, dim3(kgrid(len), K), 256, 0, ex, kseg(nu, np, K, 3), a, x, y);
+}
+template <class S, class D>
+void kadd_convert(const Exec& ex, size_t nu, size_t np, int K, const KCoefs& a, const S* x, D* y) {
+  SK_REQUIRE(K >= 1 && K <= kMaxRhs, STOKES_ERR_ARG, "kadd_convert: 1 to 8 right-hand sides");
+  const size_t len = seglen(nu, np, 3);
+  ProfScope ps(ex, STOKES_KERNEL_BLAS1, (double)(sizeof(S) + 2 * sizeof(D)) * K * len);
+  launch_dep(k_kconvert<S, D, true>, dim3(kgrid(len), K), 256, 0, ex, kseg(nu, np, K, 3), a, x, y);
+}
+
 template <class T>
 void kcg_update(const Exec& ex, const DotScratch& ds, size_t n, int K, const KCoefs& a, const T* d, T* x, const T* q,
                 T* r, double* rr) {
@@ -327,6 +356,8 @@ void ksub(const Exec& ex, int K, double* out, const double* a, const double* b) 
   SK_CHECK_LAUNCH();
 }
 
+template void kconvert<double, float>(const Exec&, size_t, size_t, int, const KCoefs&, const double*, float*);
+template void kadd_convert<float, double>(const Exec&, size_t, size_t, int, const KCoefs&, const float*, double*);
 #define SK_INSTK(T)                                                                                                  \
   template void kdot<T>(const Exec&, const DotScratch&, size_t, size_t, int, int, const T*, const T*, double*);     \
   template void kaxpby<T>(const Exec&, size_t, size_t, int, int, const KCoefs&, const T*, const KCoefs&, T*);      \

@@ -1034,21 +1034,31 @@ static void method2(stokes_ctx& c, const T* rF, const T* rg, T* dU, T* dP, doubl
 // ---------------------------------------------------------------------------
 // defect correction on the FP64 residual of the full system
 // ---------------------------------------------------------------------------
+// Inner FP32 work runs on the residual times a power of two that takes its norm
+// to [1, 2), undone exactly on the way back: sums of squares in FP32 pairs
+// overflow from a norm of 1.8e19 on and lose their low parts below about 1e-15.
+static double unit_scale(double norm) {
+  if (!(norm > 0.0) || !std::isfinite(norm)) return 1.0;
+  return std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(norm))));
+}
+
+// norm: of [rF; rg]
 template <class T>
-static void correction(stokes_ctx& c, const double* rF, const double* rg, double* U, double* P, double eta,
-                       double tol_in) {
+static void correction(stokes_ctx& c, const double* rF, const double* rg, double norm, double* U, double* P,
+                       double eta, double tol_in) {
   NvtxRange range(std::is_same<T, float>::value ? "correction pass (FP32)" : "correction pass (FP64)");
   const size_t nv = nvel(c), np = npres(c);
   Tmp<T> dU(c.pool, nv), dP(c.pool, np);
   const T* rFt;
   const T* rgt;
   Tmp<T> rF32(c.pool, std::is_same<T, double>::value ? 1 : nv), rg32(c.pool, std::is_same<T, double>::value ? 1 : np);
+  const double scale = std::is_same<T, double>::value ? 1.0 : unit_scale(norm);
   if constexpr (std::is_same<T, double>::value) {
     rFt = rF;
     rgt = rg;
   } else {
-    convert<double, float>(c.ex, nv, rF, rF32);
-    convert<double, float>(c.ex, np, rg, rg32);
+    convert<double, float>(c.ex, nv, rF, rF32, scale);
+    convert<double, float>(c.ex, np, rg, rg32, scale);
     rFt = rF32;
     rgt = rg32;
   }
@@ -1056,8 +1066,8 @@ static void correction(stokes_ctx& c, const double* rF, const double* rg, double
     method2<T>(c, rFt, rgt, dU, dP, eta, tol_in);
   else
     method1<T>(c, rFt, rgt, dU, dP, eta, tol_in);
-  add_convert<T, double>(c.ex, nv, dU, U);
-  add_convert<T, double>(c.ex, np, dP, P);
+  add_convert<T, double>(c.ex, nv, dU, U, 1.0 / scale);
+  add_convert<T, double>(c.ex, np, dP, P, 1.0 / scale);
 }
 
 static int read_flag(stokes_ctx& c) {
@@ -1151,9 +1161,9 @@ static int solve_reduced(stokes_ctx& c, const double* F, const double* g, double
       double eta = passes ? std::max(c.opt.pass_tol, 0.5 * tol / rel) : std::max(0.5 * tol / rel, 1e-13);
       double tin = passes ? std::max(c.opt.inner_tol, c.opt.pass_tol / 30.0) : c.opt.inner_tol;
       if (c.mixed)
-        correction<float>(c, rF, rg, U, P, eta, tin);
+        correction<float>(c, rF, rg, rel * normFg, U, P, eta, tin);
       else
-        correction<double>(c, rF, rg, U, P, eta, tin);
+        correction<double>(c, rF, rg, rel * normFg, U, P, eta, tin);
     }
    } catch (const Error& e) {
     // a non-finite residual after a flagged breakdown is the breakdown
@@ -1744,25 +1754,34 @@ static void full_residual_k(stokes_ctx& c, int K, const double* F, const double*
   c.sc.give(K);
 }
 
+// norm[k]: of R_k
 template <class T>
-static void correction_k(stokes_ctx& c, int K, const double* R, double* X, const double* eta, double tol_in,
-                         unsigned live, int* its) {
+static void correction_k(stokes_ctx& c, int K, const double* R, const double* norm, double* X, const double* eta,
+                         double tol_in, unsigned live, int* its) {
   NvtxRange range(std::is_same<T, float>::value ? "lockstep correction pass (FP32)" : "lockstep correction pass (FP64)");
-  const size_t KN = (size_t)K * (nvel(c) + npres(c));
+  const size_t nv = nvel(c), np = npres(c), KN = (size_t)K * (nv + np);
   Tmp<T> dX(c.pool, KN);
   Tmp<T> R32(c.pool, std::is_same<T, double>::value ? 1 : KN);
   const T* Rt;
+  KCoefs scale, back;  // per system (see unit_scale)
   if constexpr (std::is_same<T, double>::value) {
     Rt = R;
   } else {
-    convert<double, float>(c.ex, KN, R, R32);
+    for (int k = 0; k < K; ++k) {
+      scale.c[k] = unit_scale(norm[k]);
+      back.c[k] = 1.0 / scale.c[k];
+    }
+    kconvert<double, float>(c.ex, nv, np, K, scale, R, R32);
     Rt = R32;
   }
   if (c.opt.method == STOKES_METHOD_COUPLED)
     method2_k<T>(c, K, Rt, dX, eta, tol_in, live, its);
   else
     method1_k<T>(c, K, Rt, dX, eta, tol_in, live, its);
-  add_convert<T, double>(c.ex, KN, dX, X);
+  if constexpr (std::is_same<T, double>::value)
+    add_convert<double, double>(c.ex, KN, dX, X);
+  else
+    kadd_convert<float, double>(c.ex, nv, np, K, back, dX, X);
 }
 
 // K systems K [U_k; P_k] = [F_k; g_k] in the reduced spaces (as
@@ -1811,7 +1830,7 @@ static void solve_reduced_k(stokes_ctx& c, int K, const double* F, const double*
   try {
     for (int pass = 0; pending; ++pass) {
       full_residual_k(c, K, F, gp, X, R, normFg, rel);
-      double eta[kMaxRhs] = {};
+      double eta[kMaxRhs] = {}, norm[kMaxRhs] = {};
       const bool passes = c.opt.pass_schedule == 1 || (c.opt.pass_schedule == 0 && c.mixed);
       for (int k = 0; k < K; ++k) {
         if (!has_bit(pending, k)) continue;
@@ -1826,13 +1845,14 @@ static void solve_reduced_k(stokes_ctx& c, int K, const double* F, const double*
           pending &= ~(1u << k);
         }
         eta[k] = passes ? std::max(c.opt.pass_tol, 0.5 * tol / rel[k]) : std::max(0.5 * tol / rel[k], 1e-13);
+        norm[k] = rel[k] * normFg[k];
       }
       if (!pending) break;
       const double tin = passes ? std::max(c.opt.inner_tol, c.opt.pass_tol / 30.0) : c.opt.inner_tol;
       if (c.mixed)
-        correction_k<float>(c, K, R, X, eta, tin, pending, its);
+        correction_k<float>(c, K, R, norm, X, eta, tin, pending, its);
       else
-        correction_k<double>(c, K, R, X, eta, tin, pending, its);
+        correction_k<double>(c, K, R, norm, X, eta, tin, pending, its);
     }
   } catch (const Error& e) {
     if (e.status == STOKES_ERR_NAN && (read_flag(c) & 1))
