@@ -603,9 +603,10 @@ template <class T> void prolong_add_split(const Exec& ex, const Csr& P, int nr, 
                                           const SplitMap& sm);
 // FP32 P2 transfers without matrices (transfer.cu), nf and nc cubes per side,
 // nr = 3 component-major or 12 interleaved components, the fine vector
-// parity-split numbered if sm: y += P x; y = R x (false unless nf = 2 nc)
+// parity-split numbered if sm: y += P x; y = R x (where restrict_p2_fits)
 void prolong_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* y, bool il, const SplitMap* sm);
-bool restrict_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* y, bool il, const SplitMap* sm);
+bool restrict_p2_fits(int nf, int nc, bool il);
+void restrict_p2(const Exec& ex, int nc, int nr, const float* x, float* y, bool il, const SplitMap* sm);
 // [nr][rows] (natural) <-> [nr][rows] (split-numbered), or with il the
 // interleaved copies to / from split numbering
 template <class T> void to_split(const Exec& ex, size_t rows, int nr, const T* src, T* dst, bool il,

@@ -403,9 +403,10 @@ static double transfer_bytes(const stokes_ctx& c, int l, int nr, int fine_stream
   return 4.0 * nr * ((double)c.lv[l].nvi * fine_streams + c.lv[l + 1].nvi);
 }
 static bool restrict_p2_level(stokes_ctx& c, int l, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
-  if (c.lv[l].n != 2 * c.lv[l + 1].n) return false;
+  if (!restrict_p2_fits(c.lv[l].n, c.lv[l + 1].n, il)) return false;
   ProfScope ps(c.ex, STOKES_KERNEL_TRANSFER, transfer_bytes(c, l, nr, 1));
-  return restrict_p2(c.ex, c.lv[l].n, c.lv[l + 1].n, nr, x, y, il, sm);
+  restrict_p2(c.ex, c.lv[l + 1].n, nr, x, y, il, sm);
+  return true;
 }
 static void prolong_p2_level(stokes_ctx& c, int l, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
   ProfScope ps(c.ex, STOKES_KERNEL_TRANSFER, transfer_bytes(c, l, nr, 2));

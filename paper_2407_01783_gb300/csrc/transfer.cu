@@ -251,12 +251,13 @@ __global__ void __launch_bounds__(256) k_restrict_p2(const RestrictArgs a, const
     y[blockIdx.z * ys + row] = sum([](const V& v) { return v; });
 }
 
-bool restrict_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
-  // Component-major gathers are 4 words apart in x: above 32 cubes the CSR
-  // product (several lanes per row) is faster, below it its index loads cost
-  // more than the gathers. us at 8^3, 24^3, 40^3, 48^3: 2.9, 3.9, 10.3, 16.2
-  // against 3.3, 4.5, 9.1, 13.7. Interleaved rows are contiguous: always.
-  if (nf != 2 * nc || (!il && nf > 32)) return false;
+// Nested levels only. Component-major gathers are 4 words apart in x: above 32
+// cubes the CSR product (several lanes per row) is faster, below it its index
+// loads cost more than the gathers. us at 8^3, 24^3, 40^3, 48^3: 2.9, 3.9, 10.3,
+// 16.2 against 3.3, 4.5, 9.1, 13.7. Interleaved rows are contiguous: always.
+bool restrict_p2_fits(int nf, int nc, bool il) { return nf == 2 * nc && (il || nf <= 32); }
+
+void restrict_p2(const Exec& ex, int nc, int nr, const float* x, float* y, bool il, const SplitMap* sm) {
   RestrictArgs a = restrict_args(nc);
   a.split = sm ? 1 : 0;
   if (sm) a.sm = *sm;
@@ -267,7 +268,6 @@ bool restrict_p2(const Exec& ex, int nf, int nc, int nr, const float* x, float* 
     launch_dep(k_restrict_p2<12, true>, dim3(cdiv(3LL * rows, 32), 8), 256, 0, ex, a, x, xs, y, ys);
   else throw Error(STOKES_ERR_ARG, "P2 transfer: 3 component-major or 12 interleaved components");
   SK_CHECK_LAUNCH();
-  return true;
 }
 
 }  // namespace sk
