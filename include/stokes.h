@@ -96,7 +96,9 @@ typedef struct {
   int profile;           /* 1: count launches and time every kernel class with CUDA
                             events; 2 + k: count all, time only class k
                             (STOKES_KERNEL_*); 0: off */
-  int spmv_group;        /* threads per sparse row: 0 autotune, else 1..32 */
+  int spmv_group;        /* threads per row of CSR and BSR3 products: 0 autotune,
+                            else 1..32 (products from stencil storage or element
+                            by element split rows by their own rules) */
   int schur_inner_iters; /* > 0 (default 2): the solve inside C runs exactly this
                             many PCG iterations with no convergence test (no
                             host synchronisation; the outer CG is flexible);
@@ -202,9 +204,15 @@ stokes_status stokes_setup(int n, const double* vertices, double mu, double dt,
 /* Solve for (u, p). f: device [(2n+1)^3][3] nodal body force (the load is
  * F = M_V f_h on interior rows). g: device [(n+1)^3] pressure load or NULL
  * (zero); sum(g) must vanish (else STOKES_ERR_INCOMPATIBLE_RHS). tol: target
- * for the true relative residual of the full system. u: device
- * [(2n+1)^3][3] (boundary rows written as 0). p: device [(n+1)^3] with
- * int p_h = 0. info may be NULL. */
+ * for the true relative residual of the full system, one norm of
+ * [F - A U + B^T P; g - B U] over that of [F; g]. What is left in g - B U moves
+ * the pressure far more than the momentum rows do (by about h / dt, more on
+ * single modes): at tol the velocity is accurate to some 10 tol, the pressure
+ * to between tol and some 10^2.5 tol for dt from 1e-2 to 1e-4 (largest seen at
+ * 1e-12, mixed precision, N(0,1) forces: 1e-9 of |p|, 7e-8 of its rms at a
+ * node), and two solutions that differ in rounding only may differ by as much.
+ * u: device [(2n+1)^3][3] (boundary rows written as 0). p: device [(n+1)^3]
+ * with int p_h = 0. info may be NULL. */
 stokes_status stokes_solve(stokes_ctx* ctx, const double* f, const double* g,
                            double tol, double* u, double* p, stokes_info* info);
 
