@@ -121,12 +121,19 @@ struct ElNodes {
 };
 
 // Strain-form result y (edges: a quarter of it) of one tetrahedron for nodal
-// values u (vertices, then edges), geometry g and w; mu the viscosity.
-__device__ __forceinline__ void el_strain_tet(const float (&u)[10][3], float (&y)[10][3], const float (&g)[3][3],
+// values u (vertices, then edges), geometry g and w; mu the viscosity. Gradients
+// and all but the row sums of the mass matrix (-21 and 84 of 420) act on the
+// differences to the mean r of the edge values: sums of near-equal numbers and
+// their cancellation in the gradients are what costs FP32 its last bits.
+__device__ __forceinline__ void el_strain_tet(float (&u)[10][3], float (&y)[10][3], const float (&g)[3][3],
                                               float w, float mu) {
   float H[4][3][3];  // H[k][p][c] = d_p u_c at vertex k (scaled)
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
+    const float r =
+        (((u[6][c] + u[7][c]) + (u[5][c] + u[8][c])) + (u[4][c] + u[9][c])) * (float)(1.0 / 6.0);
+#pragma unroll
+    for (int a = 0; a < 10; ++a) u[a][c] -= r;
     float D[4][4];
 #pragma unroll
     for (int m = 0; m < 4; ++m)
@@ -156,13 +163,13 @@ __device__ __forceinline__ void el_strain_tet(const float (&u)[10][3], float (&y
     const float V = (u[0][c] + u[1][c]) + (u[2][c] + u[3][c]);
     const float vs = V - 6.f * S, es = 4.f * S - 1.5f * V;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) y[m][c] = w * (vs + 5.f * u[m][c] + 2.f * E[m]);
+    for (int m = 0; m < 4; ++m) y[m][c] = w * (vs + 5.f * u[m][c] + 2.f * E[m] - 21.f * r);
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = a + 1; b < 4; ++b) {
         const int e = el_edge(a, b);  // the opposite edge is 5 - e
-        y[4 + e][c] = w * (es + 4.f * u[4 + e][c] - 2.f * u[9 - e][c] + 0.5f * (u[a][c] + u[b][c]));
+        y[4 + e][c] = w * (es + 4.f * u[4 + e][c] - 2.f * u[9 - e][c] + 0.5f * (u[a][c] + u[b][c]) + 21.f * r);
       }
   }
   // strain at the vertices, weighted by the P1 mass: T[k] = mu (S[k] + sum_l S[l])
@@ -246,10 +253,12 @@ constexpr int kElBlock = 192;  // 32 cubes x 6 tetrahedra
 // against the symmetric storage it replaced (2.8 TB/s on 446 MB at 48^3):
 // 12^3 7.6 us (16), 25^3 11 (31), 33^3 17 (60), 48^3 40 (165), 64^3 87 (352),
 // 96^3 289 (1267).
-// Error against FP64 over n = 2..96, mu dt from 1e-8 to 1e-2: N(0,1) vectors
-// 5.0e-8..7.0e-8 relative (the FP32 blocks: 6.3e-8..7.5e-8); smooth vectors
-// 6.4e-6 against 1.9e-5 where the stiffness dominates (96^3, mu = 1, dt = 1e-2),
-// 5.7e-8 against 4.8e-8 where the mass does (mu = dt = 1e-4).
+// Error against FP64 over n = 12..96, (mu, dt) from (1e-6, 1e-2) to (1, 1e-2):
+// N(0,1) vectors 5.1e-8..6.8e-8 relative (the FP32 blocks: 6.3e-8..7.5e-8);
+// smooth vectors 4.3e-8 where the mass dominates (4.8e-8), 2.9e-7 at 96^3, mu = 1
+// (1.9e-5). Without the differences to the mean, which cost 0.2 of 45.4 us at
+// 48^3 and 1.9 of 290.9 at 96^3 (with events around the launches): 5.5e-8..7.0e-8,
+// 5.6e-8, 1.1e-5.
 __global__ void __launch_bounds__(kElBlock, 4) k_el_strain(int n, const float* __restrict__ G, float mu,
                                                        const float* __restrict__ x, size_t xs,
                                                        float* __restrict__ part) {

@@ -96,3 +96,23 @@ def test_stencil_products_across_warp_splits(n):
         for c in range(comps):
             assert np.linalg.norm(y[c] - M @ x[c]) <= 1e-14 * np.linalg.norm(abs(M) @ abs(x[c]))
     S.close()
+
+
+@pytest.mark.parametrize("n", [5, 9, 13])
+def test_fp32_strain_product_of_smooth_vectors(n):
+    """Where the mass term dominates, a smooth vector leaves no cancellation to
+    hide behind: the error stays below that of the product with the matrix
+    blocks rounded to FP32 (4.8e-8, about 0.8 units of rounding)."""
+    sk = gpu_module()
+    mu = dt = 1e-4
+    V = wl.kuhn_vertices(n, 0.16, 7)
+    S = sk.Stokes(n, V, mu, dt, 0.0, sk.stokes_default_options(precision=1))
+    orc = StokesSystem(KuhnMesh(n, V), mu, dt)
+    t = np.arange(1, 2 * n) / (2 * n)
+    z, y, x = np.meshgrid(t, t, t, indexing="ij")
+    s = np.sin(np.pi * x) * np.sin(np.pi * y) * np.sin(np.pi * z)
+    v = np.stack([s, 2 * s * (1 + x), -s * (1.5 + y)], axis=-1).ravel().astype(np.float32).astype(np.float64)
+    got = aos(host(S.apply("A_F32", cuda(soa(v)), v.size)))
+    want = orc.A @ v
+    assert np.linalg.norm(got - want) <= 0.8 * 2.0 ** -24 * np.linalg.norm(want)
+    S.close()
