@@ -294,6 +294,14 @@ typedef enum {
   STOKES_OP_BT_F32 = 21,      /* y = B^T x, likewise                          */
   STOKES_OP_PROLONG_P2_F32 = 22,  /* as PROLONG_P2 in FP32, likewise        */
   STOKES_OP_RESTRICT_P2_F32 = 23, /* as RESTRICT_P2 in FP32, likewise       */
+  STOKES_OP_VCYCLE_VEL_F32 = 24,  /* as VCYCLE_VEL in FP32, likewise        */
+  STOKES_OP_SCHUR_PREC_F32 = 25,  /* as SCHUR_PREC in FP32, likewise        */
+  /* added to A_F32, B_F32, BT_F32, VCYCLE_VEL_F32 or SCHUR_PREC_F32: four
+   * vectors one after another in x and y, as the lockstep solves compute them.
+   * A: x = x_0..x_3, b_0..b_3, y = A x_k, b_k - A x_k, then the four x_k . A x_k;
+   * B: x = x_0..x_3, b_0..b_3, y = b_k - B x_k;
+   * BT: x = x_0..x_3, b_0..b_3, y = b_k - Lambda_V^{-1} B^T x_k               */
+  STOKES_OP_X4 = 64,
   STOKES_OP_VCYCLE_VEL = 18   /* y = the configured velocity preconditioner
                                  (vcycles V-cycles of A~_{vel_prec}) applied
                                  to x, from level 0                          */

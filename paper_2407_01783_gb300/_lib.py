@@ -24,7 +24,8 @@ PRECISION_FP64, PRECISION_MIXED = 0, 1
 OP = dict(A=0, A3=1, B=2, BT=3, MQ=4, LQ=5, KQ=6, LUMPED_INV=7, VCYCLE_A3=8, VCYCLE_KQ=9,
           SCHUR_PREC=10, SCHUR=11, AGAMMA=12, PROLONG_P2=13, RESTRICT_P2=14, PROLONG_P1=15,
           LOAD=16, A_DF=17, VCYCLE_VEL=18, A_F32=19, B_F32=20,
-          BT_F32=21, PROLONG_P2_F32=22, RESTRICT_P2_F32=23)
+          BT_F32=21, PROLONG_P2_F32=22, RESTRICT_P2_F32=23, VCYCLE_VEL_F32=24, SCHUR_PREC_F32=25,
+          A_F32_X4=64 + 19, B_F32_X4=64 + 20, BT_F32_X4=64 + 21, VCYCLE_VEL_F32_X4=64 + 24, SCHUR_PREC_F32_X4=64 + 25)
 MAT = dict(A=0, A3=1, B=2, BT=3, MQ=4, LQ=5, KQ=6, LUMPED=7, AV=8)
 KERNEL = dict(SPMM_A3=0, SPMV_A=1, B=2, BT=3, SPMV_P1=4, TRANSFER=5, BLAS1=6, OTHER=7,
               SPMM_A3_COARSE=8, RESIDUAL=9, COARSE_CYCLE=10)

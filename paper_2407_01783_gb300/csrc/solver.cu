@@ -1992,6 +1992,35 @@ int adjoint_context(stokes_ctx* cp, const double* dJdu, const double* dJdp, doub
 // ---------------------------------------------------------------------------
 // operator access for tests (FP64)
 // ---------------------------------------------------------------------------
+// STOKES_OP_X4: the FP32 building blocks of the lockstep solves, four systems
+static void apply_lockstep(stokes_ctx& c, int op, const double* x, double* y) {
+  SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 operators need a mixed-precision context");
+  constexpr int K = kLockstep;
+  const size_t nv = nvel(c), np = npres(c), Kv = K * nv, Kp = K * np;
+  const bool a = op == STOKES_OP_A_F32, b = op == STOKES_OP_B_F32, bt = op == STOKES_OP_BT_F32;
+  const bool pressures = op == STOKES_OP_SCHUR_PREC_F32;
+  SK_REQUIRE(a || b || bt || pressures || op == STOKES_OP_VCYCLE_VEL_F32, STOKES_ERR_ARG, "no such lockstep operator");
+  const size_t nx = a ? 2 * Kv : (b || bt ? Kv + Kp : (pressures ? Kp : Kv));
+  const size_t ny = a ? 2 * Kv : (b || pressures ? Kp : Kv);
+  Tmp<float> xf(c.pool, nx), yf(c.pool, ny);
+  convert<double, float>(c.ex, nx, x, xf);
+  const float* xs = xf;
+  float* ys = yf;
+  if (a) {
+    bsr3_apply_dot_k<float>(c.ex, c.A, K, xs, ys, c.ds, y + ny);
+    bsr3_apply_k<float>(c.ex, c.A, K, xs, ys + Kv, xs + Kv);
+  } else if (b) {
+    b_apply_k<float>(c, K, xs, ys, xs + Kv, -1.0);
+  } else if (bt) {
+    bt_apply_k<float>(c, K, xs, ys, (const float*)c.lumped_inv32, xs + Kp, -1.0);
+  } else if (pressures) {
+    cprec_k<float>(c, K, xs, ys);
+  } else {
+    vcycles<float>(c, velocity_cycle(c), xs, ys, std::max(1, c.opt.vcycles), K);
+  }
+  convert<float, double>(c.ex, ny, yf, y);
+}
+
 void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* y) {
   stokes_ctx& c = *cp;
   SK_REQUIRE(level >= 0 && level < (int)c.lv.size(), STOKES_ERR_ARG, "level out of range");
@@ -2000,6 +2029,11 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       op != STOKES_OP_RESTRICT_P2 && op != STOKES_OP_PROLONG_P1)
     SK_REQUIRE(level == 0, STOKES_ERR_ARG, "operator defined on level 0 only");
   const size_t np = npres(c), nv = nvel(c);
+  if (op & STOKES_OP_X4) {
+    apply_lockstep(c, op & ~STOKES_OP_X4, x, y);
+    host_sync(c);
+    return;
+  }
   switch (op) {
     case STOKES_OP_A: bsr3_apply<double>(c.ex, c.A, x, y, nullptr); break;
     case STOKES_OP_A3: spmv_store<double>(c.ex, L.A3, 3, x, y, STOKES_KERNEL_SPMM_A3); break;
@@ -2077,6 +2111,18 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
       if (div) b_apply<float>(c.ex, c.B, xf, yf, (const float*)nullptr, 1.0);
       else bt_apply<float>(c.ex, c.Bt, xf, yf, (const float*)nullptr, (const float*)nullptr, 1.0);
       convert<float, double>(c.ex, ny, yf, y);
+      break;
+    }
+    case STOKES_OP_VCYCLE_VEL_F32:
+    case STOKES_OP_SCHUR_PREC_F32: {
+      SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 preconditioners need a mixed-precision context");
+      const bool vel = op == STOKES_OP_VCYCLE_VEL_F32;
+      const size_t len = vel ? nv : np;
+      Tmp<float> xf(c.pool, len), yf(c.pool, len);
+      convert<double, float>(c.ex, len, x, xf);
+      if (vel) vcycles<float>(c, velocity_cycle(c), xf, yf, std::max(1, c.opt.vcycles));
+      else cprec<float>(c, xf, yf);
+      convert<float, double>(c.ex, len, yf, y);
       break;
     }
     case STOKES_OP_PROLONG_P2_F32:
