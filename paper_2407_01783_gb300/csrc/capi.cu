@@ -400,25 +400,36 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
       c.B.v32 = f32_copy(c, c.B.v64, 3 * (size_t)c.B.nnz);
       c.Bt.v32 = f32_copy(c, c.Bt.v64, 3 * (size_t)c.Bt.nnz);
     }
-    c.MQ.v32 = f32_copy(c, c.MQ.v64, c.MQ.nnz);
-    c.LQ.v32 = f32_copy(c, c.LQ.v64, c.LQ.nnz);
+    // CSR copies likewise: not of matrices whose every product reads the stencil
+    // storage, nor of transfers that run without their matrix (the cooperative
+    // coarse kernel reads CSR throughout)
+    auto csr32 = [&](Csr& m) {
+      if (!m.st || m.rows < m.st_min_single || c.opt.coarse_kernel) m.v32 = f32_copy(c, m.v64, m.nnz);
+    };
+    csr32(c.MQ);
+    csr32(c.LQ);
     c.lumped_inv32 = f32_copy(c, c.lumped_inv64, L0.nvi);
     c.MQ_dinv32 = f32_copy(c, c.MQ_dinv64, L0.np);
     if (c.MV.v64) {
-      c.MV.v32 = f32_copy(c, c.MV.v64, c.MV.nnz);
+      csr32(c.MV);
       c.MV_dinv32 = f32_copy(c, c.MV_dinv64, c.MV.rows);
     }
-    for (Level& L : c.lv) {
-      L.A3.v32 = f32_copy(c, L.A3.v64, L.A3.nnz);
-      L.KQ.v32 = f32_copy(c, L.KQ.v64, L.KQ.nnz);
+    for (size_t l = 0; l < c.lv.size(); ++l) {
+      Level& L = c.lv[l];
+      csr32(L.A3);
+      csr32(L.KQ);
       L.A3_dinv32 = f32_copy(c, L.A3_dinv64, L.A3.rows);
       L.KQ_dinv32 = f32_copy(c, L.KQ_dinv64, L.KQ.rows);
       if (L.AV.v64) {
         L.AV.v32 = L.AV.v64 == c.A.v64 ? c.A.v32 : f32_copy(c, L.AV.v64, 9 * (size_t)L.AV.nnz);
         L.AV_dinv32 = f32_copy(c, L.AV_dinv64, 3 * (size_t)L.AV.rows);
       }
-      for (Csr* t : {&L.P2, &L.R2, &L.P1, &L.R1})
-        if (t->v64) t->v32 = f32_copy(c, t->v64, t->nnz);
+      if (l + 1 == c.lv.size()) continue;
+      const bool matrices = c.opt.format == 1 || c.opt.coarse_kernel;
+      if (matrices) L.P2.v32 = f32_copy(c, L.P2.v64, L.P2.nnz);
+      if (matrices || !restrict_p2_fits(L.n, c.lv[l + 1].n, false)) L.R2.v32 = f32_copy(c, L.R2.v64, L.R2.nnz);
+      L.P1.v32 = f32_copy(c, L.P1.v64, L.P1.nnz);
+      L.R1.v32 = f32_copy(c, L.R1.v64, L.R1.nnz);
     }
     for (auto& so : c.stencils) so->v32 = f32_copy(c, so->v64, so->total);
     if (c.symA) {
@@ -440,8 +451,9 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
       return;
     }
     if (m.st && m.rows >= m.st_min_single) return;  // its products read the stencil storage
+    if (c.mixed && !m.v32) return;                  // no FP32 product reads it
     Csr probe = m;
-    if (c.mixed && m.v32) probe.v64 = nullptr;
+    if (c.mixed) probe.v64 = nullptr;
     autotune_group(c.ex, probe, nr, kind, k);
     m.group = probe.group;
     m.group4 = probe.group4;

@@ -599,8 +599,7 @@ template <class T> bool stencil_in_use(const Csr& m, bool il);
 // vector: y += P x with the rows of P mapped by sm
 template <class T> void restrict_split(const Exec& ex, const Csr& R, int nr, const T* x, T* y, bool il,
                                       const SplitMap& sm);
-template <class T> void prolong_add_split(const Exec& ex, const Csr& P, int nr, const T* x, T* y, bool il,
-                                          const SplitMap& sm);
+void prolong_add_split(const Exec& ex, const Csr& P, int nr, const double* x, double* y, bool il, const SplitMap& sm);
 // FP32 P2 transfers without matrices (transfer.cu), nf and nc cubes per side,
 // nr = 3 component-major or 12 interleaved components, the fine vector
 // parity-split numbered if sm: y += P x; y = R x (where restrict_p2_fits)

@@ -199,6 +199,7 @@ template <class T> static void mg_emit_cheb(stokes_ctx& c, MgProgram& P, const C
   T* xa = x;
   T* xb = xt;
   if (xzero && (steps - 1) % 2 == 1) std::swap(xa, xb);
+  SK_REQUIRE(M.template v<T>() != nullptr, STOKES_ERR_ARG, "matrix values missing for this precision");
   auto csr_step = [&](const T* xin, T* xout, double c1, double c2) {
     MgOp o;
     o.kind = 4;
@@ -245,6 +246,7 @@ template <class T> static void mg_emit_cheb(stokes_ctx& c, MgProgram& P, const C
 
 template <class T> static void mg_emit_csr(stokes_ctx& c, MgProgram& P, int kind, const Csr& M, int nr,
                                           const T* b, const T* x, T* y) {
+  SK_REQUIRE(M.template v<T>() != nullptr, STOKES_ERR_ARG, "matrix values missing for this precision");
   MgOp o;
   o.kind = kind;
   o.nr = nr;
@@ -453,13 +455,15 @@ static void vcycle(stokes_ctx& c, int which, int l, const T* b, T* x, bool xzero
     else spmv_store<T>(c.ex, which == 1 ? L.R1 : L.R2, nr, r, bc, STOKES_KERNEL_TRANSFER, il);
   };
   auto prolong_into = [&](const T* xc, T* xf) {
-    if constexpr (std::is_same<T, float>::value)
+    if constexpr (std::is_same<T, float>::value) {
       if (which != 1 && implicit_transfers(c)) {
         prolong_p2_level(c, l, nr, xc, xf, il, split ? &sm : nullptr);
         return;
       }
-    if (split) prolong_add_split<T>(c.ex, L.P2, nr, xc, xf, il, sm);
-    else spmv_add<T>(c.ex, which == 1 ? L.P1 : L.P2, nr, xc, xf, STOKES_KERNEL_TRANSFER, il);
+    } else {  // (a split level has stencil storage, so in FP32 the transfer above)
+      if (split) return prolong_add_split(c.ex, L.P2, nr, xc, xf, il, sm);
+    }
+    spmv_add<T>(c.ex, which == 1 ? L.P1 : L.P2, nr, xc, xf, STOKES_KERNEL_TRANSFER, il);
   };
   if (l == 0 && K == 1 && coarse_kernel_ok(c, which)) {
     MgProgram* P = mg_program<T>(c, which);

@@ -1116,8 +1116,8 @@ void restrict_split(const Exec& ex, const Csr& R, int nr, const T* x, T* y, bool
     launch(ex, R, SH_CSR, x, WithColMap<EpiStore<T, NR>>{{y, (size_t)R.rows}, sm}, R.group);
   });
 }
-template <class T>
-void prolong_add_split(const Exec& ex, const Csr& P, int nr, const T* x, T* y, bool il, const SplitMap& sm) {
+void prolong_add_split(const Exec& ex, const Csr& P, int nr, const double* x, double* y, bool il, const SplitMap& sm) {
+  using T = double;
   require_il(nr, il);
   ProfScope ps(ex, STOKES_KERNEL_TRANSFER, prod_bytes(P, sizeof(T), nr, nr, 1));
   with_nr(nr, [&](auto NRc) {
@@ -1424,7 +1424,6 @@ void autotune_group(const Exec& ex, Csr& m, int nr, int kind, int k) {
                                    double, double, int, int);                                          \
   template bool stencil_in_use<T>(const Csr&, bool);                                                     \
   template void restrict_split<T>(const Exec&, const Csr&, int, const T*, T*, bool, const SplitMap&);   \
-  template void prolong_add_split<T>(const Exec&, const Csr&, int, const T*, T*, bool, const SplitMap&);                                                                     \
   template void bsr3_apply<T>(const Exec&, const Csr&, const T*, T*, const T*, int);                          \
   template void bsr3_cheb<T>(const Exec&, const Csr&, const T*, const T*, T*, T*, const T*, double, double, int); \
   template void b_apply<T>(const Exec&, const Csr&, const T*, T*, const T*, double, int);                \
