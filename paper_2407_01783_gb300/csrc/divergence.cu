@@ -83,13 +83,18 @@ DivOp* div_from_csr(const Exec& ex, Arena& ar, const StencilTables* st, int n, c
 
 // y = b + alpha B x for K right-hand sides. A block takes 32 vertices, its warp
 // w the entries w, w + 8, ... of each: eight times the loads in flight of a
-// thread per row, which small meshes need (17 576 rows at 25^3).
+// thread per row, which small meshes need (17 576 rows at 25^3). A vertex knows
+// its interior offsets per axis as bits and leaves the other entries out of its
+// sum: their weight is 0, but what is read for them is another node's value, which
+// may be an infinity.
+__host__ __device__ constexpr unsigned div_bit(int axis, int d) { return 1u << (5 * axis + d + 2); }
 template <int E, int N, int K, class T> struct DivRow {  // entries E, E + 8, ... (N of them), all loads issued first
+  using Seq = std::make_integer_sequence<int, N>;
   static __device__ __forceinline__ void run(const T* __restrict__ v, const T* __restrict__ x, size_t np, size_t xs,
-                                             int m, int base, int last, T* acc) {
+                                             int m, int base, int last, unsigned in, T* acc) {
     T w[N][3];
     int c[N];
-    load(std::make_integer_sequence<int, N>(), v, np, m, base, last, w, c);
+    load(Seq(), v, np, m, base, last, w, c);
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       T xv[N][3];
@@ -97,9 +102,7 @@ template <int E, int N, int K, class T> struct DivRow {  // entries E, E + 8, ..
       for (int t = 0; t < N; ++t)
 #pragma unroll
         for (int u = 0; u < 3; ++u) xv[t][u] = x[(size_t)(3 * q + u) * xs + c[t]];
-#pragma unroll
-      for (int t = 0; t < N; ++t)
-        acc[2 * q + t % 2] += w[t][0] * xv[t][0] + w[t][1] * xv[t][1] + w[t][2] * xv[t][2];
+      add(Seq(), in, w, xv, acc + 2 * q);
     }
   }
   template <int... I>
@@ -112,19 +115,30 @@ template <int E, int N, int K, class T> struct DivRow {  // entries E, E + 8, ..
                                              int& c) {
 #pragma unroll
     for (int u = 0; u < 3; ++u) w[u] = v[(size_t)(3 * F + u) * np];
-    c = min(max(base + div_d<F, 0>() + m * (div_d<F, 1>() + m * div_d<F, 2>()), 0), last);  // absent ones weigh 0
+    c = min(max(base + div_d<F, 0>() + m * (div_d<F, 1>() + m * div_d<F, 2>()), 0), last);  // (absent ones: any)
+  }
+  template <int... I>
+  static __device__ __forceinline__ void add(std::integer_sequence<int, I...>, unsigned in, const T (*w)[3],
+                                             const T (*xv)[3], T* acc) {
+    (sum<E + 8 * I>(in, w[I], xv[I], acc[I % 2]), ...);
+  }
+  template <int F>
+  static __device__ __forceinline__ void sum(unsigned in, const T* w, const T* xv, T& acc) {
+    constexpr unsigned need = div_bit(0, div_d<F, 0>()) | div_bit(1, div_d<F, 1>()) | div_bit(2, div_d<F, 2>());
+    const T s = w[0] * xv[0] + w[1] * xv[1] + w[2] * xv[2];
+    if ((in & need) == need) acc += s;
   }
 };
 template <int W, int K, class T>
 __device__ __forceinline__ void div_warp(int w, const T* __restrict__ v, const T* __restrict__ x, size_t np, size_t xs,
-                                         int m, int base, int last, T* acc) {
+                                         int m, int base, int last, unsigned in, T* acc) {
   if (w == W) {
     constexpr int N = (kDivS - W + 7) / 8;
     constexpr int H = K > 1 || sizeof(T) == 8 ? N / 2 : N;  // (registers: in two parts)
-    DivRow<W, H, K, T>::run(v, x, np, xs, m, base, last, acc);
-    if constexpr (N > H) DivRow<W + 8 * H, N - H, K, T>::run(v, x, np, xs, m, base, last, acc);
+    DivRow<W, H, K, T>::run(v, x, np, xs, m, base, last, in, acc);
+    if constexpr (N > H) DivRow<W + 8 * H, N - H, K, T>::run(v, x, np, xs, m, base, last, in, acc);
   } else if constexpr (W < 7) {
-    div_warp<W + 1, K, T>(w, v, x, np, xs, m, base, last, acc);
+    div_warp<W + 1, K, T>(w, v, x, np, xs, m, base, last, in, acc);
   }
 }
 
@@ -139,10 +153,16 @@ __global__ void __launch_bounds__(256, 4) k_div(int n, FastDiv by_v, FastDiv by_
   const int r = blockIdx.x * 32 + lane, rr = min(r, np - 1);
   const int k = by_vv.div(rr), rk = rr - k * by_vv.d, j = by_v.div(rk), i = rk - j * nv;
   const int base = (2 * i - 1) + m * ((2 * j - 1) + m * (2 * k - 1)), last = (int)xs - 1;
+  unsigned in = 0;
+#pragma unroll
+  for (int d = -2; d <= 2; ++d) {
+    const auto inside = [&](int a) { return 2 * a + d >= 1 && 2 * a + d <= m; };
+    in |= (inside(i) ? div_bit(0, d) : 0u) | (inside(j) ? div_bit(1, d) : 0u) | (inside(k) ? div_bit(2, d) : 0u);
+  }
   T acc[2 * K];  // two partial sums each
 #pragma unroll
   for (int q = 0; q < 2 * K; ++q) acc[q] = T(0);
-  div_warp<0, K, T>(w, v + rr, x, np, xs, m, base, last, acc);
+  div_warp<0, K, T>(w, v + rr, x, np, xs, m, base, last, in, acc);
 #pragma unroll
   for (int q = 0; q < K; ++q) sh[w][q][lane] = acc[2 * q] + acc[2 * q + 1];
   __syncthreads();

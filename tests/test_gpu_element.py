@@ -116,3 +116,34 @@ def test_fp32_strain_product_of_smooth_vectors(n):
     want = orc.A @ v
     assert np.linalg.norm(got - want) <= 0.8 * 2.0 ** -24 * np.linalg.norm(want)
     S.close()
+
+
+@pytest.mark.parametrize("n", [2, 5, 8])
+def test_divergence_of_non_finite_entries(n):
+    """An infinity in x reaches the rows of B that hold its node and no others
+    (rows of other nodes whose offsets leave the mesh alias it in the linear
+    index), in one system and in one of four."""
+    sk = gpu_module()
+    V = wl.kuhn_vertices(n, 0.16, 3)
+    S = sk.Stokes(n, V, 1e-2, 1e-3, 0.0, sk.stokes_default_options(precision=1))
+    orc = StokesSystem(KuhnMesh(n, V), 1e-2, 1e-3)
+    nv, npr = orc.A.shape[0], orc.B.shape[0]
+    rng = np.random.default_rng(n)
+    u = rng.standard_normal((4, nv)).astype(np.float32).astype(np.float64)
+    for node in (0, nv // 6, nv // 3 - 1):  # the first, a middle and the last interior node
+        bad = u[0].copy()
+        bad[3 * node + 1] = np.inf
+        touched = np.asarray(abs(orc.B)[:, 3 * node:3 * node + 3].sum(axis=1)).ravel() > 0
+        assert touched.any()
+        four = np.stack([soa(u[1]), soa(bad), soa(u[2]), soa(u[3])])
+        y4 = host(S.apply("B_F32_X4", cuda(np.concatenate([four.ravel(), np.zeros(4 * npr)])), 4 * npr)).reshape(4, npr)
+        finite = host(S.apply("B_F32_X4", cuda(np.concatenate([np.stack([soa(v) for v in u]).ravel(), np.zeros(4 * npr)])),
+                              4 * npr)).reshape(4, npr)
+        for op, y, good in (("B", None, None), ("B_F32", None, None), ("X4", y4[1], finite[0])):
+            if y is None:
+                y, good = (host(S.apply(op, cuda(soa(v)), npr)) for v in (bad, u[0]))
+            assert np.array_equal(y[~touched], good[~touched])
+            assert not np.isfinite(y[touched]).any()
+        for k, j in ((0, 1), (2, 2), (3, 3)):
+            assert np.array_equal(y4[k], finite[j])
+    S.close()
