@@ -1996,6 +1996,17 @@ int adjoint_context(stokes_ctx* cp, const double* dJdu, const double* dJdp, doub
 // ---------------------------------------------------------------------------
 // operator access for tests (FP64)
 // ---------------------------------------------------------------------------
+// y = M x of an exported matrix. Stencil storage multiplies absent entries by 0,
+// which carries an infinity or a NaN in x to rows that do not hold it (the solves
+// refuse such input); CSR does not.
+static void apply_scalar(stokes_ctx& c, const Csr& M, int nr, const double* x, double* y, int kind) {
+  SK_CUDA(cudaMemsetAsync(c.d_flag, 0, sizeof(int), c.ex.s));
+  count_nonfinite(c.ex, (size_t)M.cols * nr, x, c.d_flag);
+  Csr m = M;
+  if (read_flag(c) & 2) m.st = nullptr;
+  spmv_store<double>(c.ex, m, nr, x, y, kind);
+}
+
 // STOKES_OP_X4: the FP32 building blocks of the lockstep solves, four systems
 static void apply_lockstep(stokes_ctx& c, int op, const double* x, double* y) {
   SK_REQUIRE(c.mixed, STOKES_ERR_ARG, "FP32 operators need a mixed-precision context");
@@ -2040,12 +2051,12 @@ void apply_operator(stokes_ctx* cp, int op, int level, const double* x, double* 
   }
   switch (op) {
     case STOKES_OP_A: bsr3_apply<double>(c.ex, c.A, x, y, nullptr); break;
-    case STOKES_OP_A3: spmv_store<double>(c.ex, L.A3, 3, x, y, STOKES_KERNEL_SPMM_A3); break;
+    case STOKES_OP_A3: apply_scalar(c, L.A3, 3, x, y, STOKES_KERNEL_SPMM_A3); break;
     case STOKES_OP_B: b_apply<double>(c.ex, c.B, x, y, nullptr, 1.0); break;
     case STOKES_OP_BT: bt_apply<double>(c.ex, c.Bt, x, y, nullptr, nullptr, 1.0); break;
-    case STOKES_OP_MQ: spmv_store<double>(c.ex, c.MQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
-    case STOKES_OP_LQ: spmv_store<double>(c.ex, c.LQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
-    case STOKES_OP_KQ: spmv_store<double>(c.ex, L.KQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
+    case STOKES_OP_MQ: apply_scalar(c, c.MQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
+    case STOKES_OP_LQ: apply_scalar(c, c.LQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
+    case STOKES_OP_KQ: apply_scalar(c, L.KQ, 1, x, y, STOKES_KERNEL_SPMV_P1); break;
     case STOKES_OP_LUMPED_INV: {
       // y = Lambda^{-1} x per node and component
       Tmp<double> ones(c.pool, 1);

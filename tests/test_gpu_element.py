@@ -147,3 +147,24 @@ def test_divergence_of_non_finite_entries(n):
         for k, j in ((0, 1), (2, 2), (3, 3)):
             assert np.array_equal(y4[k], finite[j])
     S.close()
+
+
+@pytest.mark.parametrize("n", [2, 5, 8])
+def test_stencil_products_of_non_finite_entries(n):
+    """The same for A~_3 and the P1 operators, against their exported CSR
+    matrices."""
+    sk = gpu_module()
+    S = sk.Stokes(n, wl.kuhn_vertices(n, 0.16, 5), 1e-2, 1e-3)
+    rng = np.random.default_rng(n)
+    for op, comps in (("A3", 3), ("KQ", 1), ("MQ", 1), ("LQ", 1)):
+        rp, ci, v, shp = S.matrix(op)
+        M = to_scipy(rp, ci, v, shp)
+        x = rng.standard_normal((comps, shp[1]))
+        for node in (0, shp[1] // 2, shp[1] - 1):
+            bad = x.copy()
+            bad[0, node] = np.inf
+            y = host(S.apply(op, cuda(bad.ravel()), comps * shp[0])).reshape(comps, -1)
+            touched = np.asarray(abs(M)[:, [node]].sum(axis=1)).ravel() > 0
+            assert np.isfinite(y[1:]).all() and np.isfinite(y[0][~touched]).all()
+            assert not np.isfinite(y[0][touched]).any()
+    S.close()
