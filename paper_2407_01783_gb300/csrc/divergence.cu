@@ -6,10 +6,11 @@
 // entry (i - k) of vertex k, and consecutive nodes of one parity class meet
 // consecutive vertices, so B^T reads the same words coalesced too.
 //
-// Bound by HBM: 3 x 65 words per vertex (93 MB FP32 at 48^3, 17% less than CSR
-// with its indices) and the vectors. Against the CSR products it replaced, us at
-// 12^3, 25^3, 33^3, 48^3, 96^3: B 2.4, 4.1, 6.5, 23, 152 (3.1, 5.8, 10.6, 34,
-// 210), B^T 2.9, 3.7, 5.6, 19, 153 (2.2, 4.8, 8.4, 30, 212); 5.3 TB/s at 96^3.
+// Bound by HBM on large meshes (5.3 TB/s at 96^3), by loads in flight on small ones
+// (40% of the DRAM rate at 36^3): 3 x 65 words per vertex (93 MB FP32 at 48^3, 17%
+// less than CSR with its indices) and the vectors. Against the CSR products it replaced, us at
+// 12^3, 25^3, 33^3, 48^3, 96^3: B 2.4, 4.1, 6.5, 23, 155 (3.1, 5.8, 10.6, 34,
+// 210), B^T 2.9, 3.7, 5.6, 19, 153 (2.2, 4.8, 8.4, 30, 212).
 #include <algorithm>
 #include <utility>
 

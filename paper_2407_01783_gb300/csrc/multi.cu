@@ -8,7 +8,8 @@
 // blockIdx.y is the right-hand side, so the K systems keep their own
 // coefficients and dot products while sharing one launch. Dot products are
 // reduced in a fixed order (deterministic): per-thread sums in FP64 (FP64
-// vectors) or double-float (FP32 vectors), FP64 across threads.
+// vectors) or double-float (FP32 vectors), FP64 across threads (the squares of a CG
+// update in double-float across a warp, FP64 beyond).
 #include <algorithm>
 #include <type_traits>
 
