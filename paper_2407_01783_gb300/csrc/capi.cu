@@ -201,7 +201,10 @@ void setup_context(stokes_ctx* cp, int n, const double* Xh) {
       std::vector<cudaStream_t> s;
       std::vector<cudaEvent_t> e;
       ~Streams() {
-        for (cudaStream_t x : s) cudaStreamDestroy(x);
+        for (cudaStream_t x : s) {
+          cudaStreamSynchronize(x);  // (after an error: the caller frees what these launches write)
+          cudaStreamDestroy(x);
+        }
         for (cudaEvent_t x : e) cudaEventDestroy(x);
       }
     } side;
